@@ -108,7 +108,9 @@ typedef struct {
   int spmv_group;     /* 0: autotune/heuristic; 1..16: lanes per block row; 101..116: 100 + lanes per
                          scalar row; 301..316: 300 + lanes per block row of the 16-byte kernels on
                          the padded copy (matrices without one use the scalar-row kernel with
-                         that many lanes) (forces the product kernel of every matrix) */
+                         that many lanes); 401, 402, 404, 408: 1, 2, 5, 10 triples of lanes per block
+                         row of 3x3 blocks (other shapes by the heuristic) (forces the product
+                         kernel of every matrix) */
   int sell;           /* 0: slab products; W > 0: products with A, Shat and L use a sliced block-ELL
                          copy with rows sorted by length inside windows of W block rows
                          (W a multiple of 32, at most 1024); default 0 */

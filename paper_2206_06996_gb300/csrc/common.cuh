@@ -58,6 +58,14 @@ struct DBsr {
   // BF16 copy of val (same slab layout): when set, FP32 products read these
   // values instead (coarse AMG levels of the mixed-precision form)
   const void* hval = nullptr;
+  // the stored arrays were written before the last host synchronisation and
+  // stay as they are until the next set-up: a product launched while its
+  // predecessor drains may read them before it waits (pdl)
+  bool settled = false;
+  // rows of more than lthr blocks (build_long_rows), which a product gives a
+  // CTA each
+  const int* lrow = nullptr;
+  int nlong = 0, lthr = 0x7fffffff;
 };
 
 // Sliced block-ELL copy of a block matrix (see sell.cu): chunks of 32 block

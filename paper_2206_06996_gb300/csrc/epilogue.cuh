@@ -17,33 +17,59 @@ struct Epilogue {
   XT* dout;
   XT* xsol;
   XT alpha, beta;
+  // what the epilogue reads at (gi, o).  A product kernel loads it before its
+  // sums are done, so that these reads are in flight with the product's own
+  // instead of starting after the last multiply-add (gi is read and written
+  // by its owner only, so the early read sees what a late one would)
+  struct Operands {
+    XT p, q, t, d;
+  };
+  __device__ __forceinline__ Operands load(long long gi, long long o) const {
+    Operands v{(XT)0, (XT)0, (XT)0, (XT)0};
+    if constexpr (E == Epi::Axpby) {
+      if (z) v.p = z[gi];
+    } else if constexpr (E == Epi::Resid) {
+      v.p = z[gi];
+    } else if constexpr (E == Epi::Jacobi || E == Epi::ChebFirst) {
+      v.p = z[gi], v.q = xs[gi], v.d = dinv[o];
+    } else if constexpr (E == Epi::ScaledSub) {
+      v.p = z[gi], v.d = dinv[o];
+    } else if constexpr (E == Epi::ChebStep) {
+      v.p = r[gi], v.q = xin[gi], v.t = xsol[gi], v.d = dinv[o];
+    }
+    return v;
+  }
   template <typename AT>
-  __device__ __forceinline__ void operator()(long long gi, long long o, AT acc) const {
+  __device__ __forceinline__ void store(long long gi, AT acc, const Operands& v) const {
     if constexpr (E == Epi::Set) {
       y[gi] = (XT)acc;
     } else if constexpr (E == Epi::Axpby) {
-      XT v = alpha * (XT)acc;
-      if (z) v += beta * z[gi];
-      y[gi] = v;
+      XT w = alpha * (XT)acc;
+      if (z) w += beta * v.p;
+      y[gi] = w;
     } else if constexpr (E == Epi::Resid) {
-      y[gi] = z[gi] - (XT)acc;
+      y[gi] = v.p - (XT)acc;
     } else if constexpr (E == Epi::Jacobi) {
-      y[gi] = xs[gi] + (z[gi] - (XT)acc) * dinv[o];
+      y[gi] = v.q + (v.p - (XT)acc) * v.d;
     } else if constexpr (E == Epi::ScaledSub) {
-      y[gi] = z[gi] - (XT)acc * dinv[o];
+      y[gi] = v.p - (XT)acc * v.d;
     } else if constexpr (E == Epi::ChebFirst) {
-      const XT ri = (z[gi] - (XT)acc) * dinv[o];
+      const XT ri = (v.p - (XT)acc) * v.d;
       const XT di = alpha * ri;
       r[gi] = ri;
       dout[gi] = di;
-      y[gi] = xs[gi] + di;
+      y[gi] = v.q + di;
     } else {
-      const XT ri = r[gi] - (XT)acc * dinv[o];
-      const XT di = alpha * xin[gi] + beta * ri;
+      const XT ri = v.p - (XT)acc * v.d;
+      const XT di = alpha * v.q + beta * ri;
       r[gi] = ri;
       dout[gi] = di;
-      xsol[gi] += di;
+      xsol[gi] = v.t + di;
     }
+  }
+  template <typename AT>
+  __device__ __forceinline__ void operator()(long long gi, long long o, AT acc) const {
+    store(gi, acc, load(gi, o));
   }
 };
 

@@ -102,6 +102,37 @@ void build_sell(const DBsr<double>& M, DSell<VT>& S, DeviceArena& a, cudaStream_
 template <typename VT>
 void build_vec(DBsr<VT>& M, DeviceArena& a, cudaStream_t s);
 
+// Long rows of matrices (DBsr::lrow): those of more than max(32, 3 x the
+// mean) blocks, or of more than max(64, 8 x the mean) where the first are
+// more than one row in 512 (and 64): a CTA per row costs more than its share
+// of a lane group's waiting when many rows are long (Shat of the bench tube:
+// one row in ten, FP64 product 169 -> 323 us).  add() queues a pattern, read() waits once for all queued ones, set() gives list id to a
+// matrix with that pattern.
+class LongRows {
+ public:
+  LongRows(DeviceArena& a, cudaStream_t s);
+  int add(int nbr, long long nnzb, const int* rp);
+  void read();
+  template <typename VT>
+  void set(int id, DBsr<VT>& M) const {
+    const List& l = lists_[id];
+    M.lrow = l.rows + l.pick * l.cap;
+    M.nlong = l.n;
+    M.lthr = l.n ? l.thr[l.pick] : 0x7fffffff;
+  }
+
+ private:
+  static constexpr int kMax = 64;
+  struct List {
+    int* rows;
+    int thr[2], cap, n, pick;
+  };
+  DeviceArena& a_;
+  cudaStream_t s_;
+  int* cnt_;
+  std::vector<List> lists_;
+};
+
 // forced kernel code for every product (0: per-matrix choice)
 void set_forced_group(int code);
 int forced_group();

@@ -1,0 +1,46 @@
+// Programmatic dependent launch (option pdl): a kernel lets the next kernel
+// of the stream start as soon as all of its CTAs are running
+// (griddepcontrol.launch_dependents) and, before it reads anything an earlier
+// kernel wrote, waits for that kernel to complete with its memory visible
+// (griddepcontrol.wait).  Between the two it touches only stored matrices
+// that no kernel in flight writes.  Every kernel launched this way waits
+// itself, so a completed predecessor means that all earlier ones completed.
+// Launched without the attribute, both instructions return at once.
+//
+// The assembler and the compiler may move loads through the read-only path
+// (__ldg, const __restrict__ arguments) across the wait.  So a kernel reads
+// that way only what no kernel in flight may write (settled matrices), and
+// vectors with ordinary loads behind the wait.
+#pragma once
+#include "common.cuh"
+
+namespace scr {
+
+__device__ __forceinline__ void pdl_allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait_prev() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+extern int g_pdl;
+
+// kern<<<grid, blk, 0, s>>>(args...), with the programmatic-serialization
+// attribute when early is set (and the option pdl); kern waits in
+// griddepcontrol.wait
+template <typename... KArgs, typename... Args>
+inline void launch_early(bool early, void (*kern)(KArgs...), long long grid, int blk, cudaStream_t s, Args... args) {
+  if (early && g_pdl) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)blk);
+    cfg.dynamicSmemBytes = 0;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    SCR_CUDA(cudaLaunchKernelEx(&cfg, kern, args...));
+  } else {
+    kern<<<(unsigned)grid, blk, 0, s>>>(args...);
+  }
+}
+
+}  // namespace scr

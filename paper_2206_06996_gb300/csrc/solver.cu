@@ -346,6 +346,24 @@ struct Hierarchy {
       cinvf = ar.alloc<float>((size_t)nc * nc + 1);
       cast_d2f(cinv, cinvf, (long long)nc * nc, s);
     }
+    // long rows of the levels' operators and restrictions
+    {
+      LongRows lr(ar, s);
+      std::vector<int> ia(lv.size(), -1), ir(lv.size(), -1);
+      for (size_t l = 0; l + 1 < lv.size(); ++l) {
+        if (!lv[l].A.lrow) ia[l] = lr.add(lv[l].A.nbr, lv[l].A.nnzb, lv[l].A.rp);
+        ir[l] = lr.add(lv[l].R.nbr, lv[l].R.nnzb, lv[l].R.rp);
+      }
+      lr.read();
+      for (size_t l = 0; l + 1 < lv.size(); ++l) {
+        if (ia[l] >= 0) lr.set(ia[l], lv[l].A);
+        lv[l].Af.lrow = lv[l].A.lrow;
+        lv[l].Af.nlong = lv[l].A.nlong;
+        lv[l].Af.lthr = lv[l].A.lthr;
+        lr.set(ir[l], lv[l].R);
+        lr.set(ir[l], lv[l].Rf);
+      }
+    }
     // lane-group widths of the products on the two finest levels
     if (o.autotune) {
       for (size_t l = 0; l < lv.size() && l < 2; ++l) {
@@ -367,6 +385,7 @@ struct Hierarchy {
       }
     }
     SCR_CUDA(cudaStreamSynchronize(s));
+    settle(true);
   }
 
   // New values on the patterns of the last build: A0 has the pattern of the
@@ -382,6 +401,7 @@ struct Hierarchy {
     gsize = 0;
     const int nl = n_levels();
     if (nl == 0) return;
+    settle(false);
     lv[0].A.val = A0.val;
     lv[0].A.vdesc = A0.vdesc;
     lv[0].A.vval = A0.vval;
@@ -449,6 +469,16 @@ struct Hierarchy {
     }
     if (f32) cast_d2f(cinv, cinvf, (long long)nc * nc, s);
     SCR_CUDA(cudaStreamSynchronize(s));
+    settle(true);
+  }
+
+  // marks the levels' matrices as written (set-up synchronised) or about to
+  // be rewritten
+  void settle(bool on) {
+    for (Level& L : lv) {
+      L.A.settled = L.P.settled = L.R.settled = on;
+      L.Af.settled = L.Pf.settled = L.Rf.settled = on;
+    }
   }
 
   template <typename T>
@@ -1187,6 +1217,10 @@ struct scr_ctx {
   double *pc_r = nullptr, *pc_y = nullptr;
   LaunchCounter pc_sec;
   int pc_a_solves = 0;
+  void settle_blocks(bool on) {
+    A.settled = B.settled = C.settled = D.settled = Shat.settled = on;
+    Af.settled = Bf.settled = Cf.settled = Df.settled = on;
+  }
   scr_ctx() {
     hS.slot = 1;
     hM.slot = 2;
@@ -1752,6 +1786,7 @@ int scr_update_values(scr_handle h, const scr_bsr* A, const scr_bsr* B, const sc
     auto t0 = Clock::now();
     cudaStream_t s = h->s;
     SCR_CUDA(cudaStreamSynchronize(s));
+    h->settle_blocks(false);
     update_values(A, h->A, dev, s, "A");
     update_values(B, h->B, dev, s, "B");
     update_values(C, h->C, dev, s, "C");
@@ -1795,6 +1830,7 @@ int scr_update_values(scr_handle h, const scr_bsr* A, const scr_bsr* B, const sc
     h->hS.refresh(h->Shat, h->o, s);
     h->graph_epoch++;
     SCR_CUDA(cudaStreamSynchronize(s));
+    h->settle_blocks(true);
     h->stats.setup_ms = ms_since(t0);
   });
 }
@@ -1888,6 +1924,14 @@ int scr_setup(scr_handle h, const scr_bsr* A, const scr_bsr* B, const scr_bsr* C
       build_vec<double>(h->A, a, s);
       build_vec<double>(h->Shat, a, s);
     }
+    LongRows lr(a, s);
+    const int lA = lr.add(nv, h->A.nnzb, h->A.rp), lS = lr.add(np, h->Shat.nnzb, h->Shat.rp);
+    const int lB = lr.add(nv, h->B.nnzb, h->B.rp), lC = lr.add(np, h->C.nnzb, h->C.rp);
+    lr.read();
+    lr.set(lA, h->A);
+    lr.set(lS, h->Shat);
+    lr.set(lB, h->B);
+    lr.set(lC, h->C);
     tune_product<double>(h->A, 1, h->o, a, s);
     tune_product<double>(h->Shat, 1, h->o, a, s);
     if (f32) {
@@ -1896,6 +1940,9 @@ int scr_setup(scr_handle h, const scr_bsr* A, const scr_bsr* B, const scr_bsr* C
       h->Bf = float_copy(h->B, a, s);
       h->Cf = float_copy(h->C, a, s);
       h->Df = float_copy(h->D, a, s);
+      lr.set(lA, h->Af);
+      lr.set(lB, h->Bf);
+      lr.set(lC, h->Cf);
       if (h->o.sell) {
         build_sell<float>(h->A, h->Af_sell, a, s, h->o.sell);
         h->Af.sell = &h->Af_sell;
@@ -1956,6 +2003,7 @@ int scr_setup(scr_handle h, const scr_bsr* A, const scr_bsr* B, const scr_bsr* C
       h->rp2 = w.alloc<double>((long long)np * k + 1);
     }
     SCR_CUDA(cudaStreamSynchronize(s));
+    h->settle_blocks(true);
     h->have_block = true;
     h->stats.levels_A = h->hA.n_levels();
     h->stats.levels_S = h->hS.n_levels();
@@ -2354,6 +2402,10 @@ int mm_setup(scr_handle h, const scr_bsr* L, int dev) {
       build_sell<double>(h->L, h->L_sell, *h->mmats, s, o.sell);
       h->L.sell = &h->L_sell;
     }
+    LongRows lr(*h->mmats, s);
+    const int lL = lr.add(h->nm, h->L.nnzb, h->L.rp);
+    lr.read();
+    lr.set(lL, h->L);
     tune_product<double>(h->L, 3, o, *h->mmats, s);
     h->hM.build(h->L, 1, 3, o, false, s);
     h->mwork.reset(new DeviceArena(s));
@@ -2368,6 +2420,7 @@ int mm_setup(scr_handle h, const scr_bsr* L, int dev) {
     h->mq = w.alloc<double>(n + 1);
     h->cg = w.alloc<CgState>(1);
     SCR_CUDA(cudaStreamSynchronize(s));
+    h->L.settled = true;
     h->have_mesh = true;
     h->stats.levels_M = h->hM.n_levels();
     h->stats.mm_setup_ms = ms_since(t0);

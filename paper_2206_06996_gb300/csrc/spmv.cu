@@ -259,6 +259,54 @@ template void refresh_vec<float>(DBsr<float>&, cudaStream_t);
 template void build_vec<double>(DBsr<double>&, DeviceArena&, cudaStream_t);
 template void build_vec<float>(DBsr<float>&, DeviceArena&, cudaStream_t);
 
+// ------------------------------------------------------------ long rows
+// rows of more than thr[q] blocks, listed in rows + q cap, counted in cnt[q]
+__global__ void k_long_rows(int nbr, const int* __restrict__ rp, int thr0, int thr1, int cap, int* __restrict__ rows,
+                            int* __restrict__ cnt) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nbr) return;
+  const int k = rp[i + 1] - rp[i];
+#pragma unroll
+  for (int t = 0; t < 2; ++t)
+    if (k > (t ? thr1 : thr0)) {
+      const int q = atomicAdd(cnt + t, 1);  // any order: each row's sum is its own
+      if (q < cap) rows[t * cap + q] = i;
+    }
+}
+LongRows::LongRows(DeviceArena& a, cudaStream_t s) : a_(a), s_(s) {
+  cnt_ = a.alloc<int>(2 * kMax);
+  SCR_CUDA(cudaMemsetAsync(cnt_, 0, sizeof(int) * 2 * kMax, s));
+}
+int LongRows::add(int nbr, long long nnzb, const int* rp) {
+  const int id = (int)lists_.size();
+  if (id >= kMax) throw CudaError{cudaErrorInvalidValue, "too many long-row lists"};
+  List l;
+  const long long mean = nbr ? nnzb / nbr : 0;
+  l.thr[0] = (int)std::max<long long>(32, 3 * mean);
+  l.thr[1] = (int)std::max<long long>(64, 8 * mean);
+  l.cap = std::max(64, nbr / 512);
+  l.n = l.pick = 0;
+  l.rows = a_.alloc<int>(2 * l.cap);
+  if (nbr > 0) {
+    k_long_rows<<<ceil_div(nbr, 256), 256, 0, s_>>>(nbr, rp, l.thr[0], l.thr[1], l.cap, l.rows, cnt_ + 2 * id);
+    SCR_LAUNCH();
+    counters().launches++;
+  }
+  lists_.push_back(l);
+  return id;
+}
+void LongRows::read() {
+  int h[2 * kMax] = {};
+  SCR_CUDA(cudaMemcpyAsync(h, cnt_, sizeof h, cudaMemcpyDeviceToHost, s_));
+  SCR_CUDA(cudaStreamSynchronize(s_));
+  for (size_t i = 0; i < lists_.size(); ++i)
+    for (int t = 1; t >= 0; --t)
+      if (h[2 * i + t] <= lists_[i].cap) {
+        lists_[i].n = h[2 * i + t];
+        lists_[i].pick = t;
+      }
+}
+
 // ------------------------------------------------------------ SpMV
 // CTAs ahead for the L2 prefetch of the scalar-row kernel (0: off); set
 // from the options at scr_create.  Measured on the 616k-node tube: 128 to
@@ -305,6 +353,10 @@ static void product(int G, const DBsr<VT>& M, const XT* x, XT* y, int nrhs, cons
       H.col = M.col;
       H.val = static_cast<__nv_bfloat16*>(const_cast<void*>(M.hval));
       H.g = M.g;
+      H.settled = M.settled;
+      H.lrow = M.lrow;
+      H.nlong = M.nlong;
+      H.lthr = M.lthr;
       spmv_launch<__nv_bfloat16, XT>(G, H, x, y, nrhs, e, s);
       return;
     }
@@ -391,14 +443,25 @@ int autotune_spmv(DBsr<VT>& M, int nrhs, cudaStream_t s) {
     ep.xsol = ev + 2 * ny;
     ep.dout = y;
   }
+  // timed as in a solve, with early launches of a settled matrix
+  SCR_CUDA(cudaStreamSynchronize(s));
+  const bool was_settled = M.settled;
+  M.settled = true;
   cudaEvent_t e0, e1;
   SCR_CUDA(cudaEventCreate(&e0));
   SCR_CUDA(cudaEventCreate(&e1));
   // the scalar-row kernel with 1, 2, 4 or 8 lanes (the block-row and
   // sliced-ELL variants measured slower on the tube operators)
-  int cands[12] = {101, 102, 104, 108};
+  int cands[16] = {101, 102, 104, 108};
   int ncand = 4;
   if (M.nbr && (double)M.nnzb * M.bc / M.nbr >= 64) cands[ncand++] = 116;  // long rows
+  // triples of lanes per block row (3x3 blocks, one right-hand side)
+  if (M.br == 3 && M.bc == 3 && nrhs == 1) {
+    cands[ncand++] = 401;
+    cands[ncand++] = 402;
+    cands[ncand++] = 404;
+    if (M.nbr < 4096) cands[ncand++] = 408;
+  }
   // the 16-byte kernels on the padded copy (one right-hand side)
   if (M.vdesc && nrhs == 1) {
     cands[ncand++] = 302;
@@ -409,7 +472,7 @@ int autotune_spmv(DBsr<VT>& M, int nrhs, cudaStream_t s) {
   float best = 1e30f;
   int bestg = M.g;
   const int saved = M.g;
-  float times[12] = {};
+  float times[16] = {};
   for (int q = 0; q < ncand; ++q) {
     const int code = cands[q];
     M.g = code;
@@ -429,6 +492,7 @@ int autotune_spmv(DBsr<VT>& M, int nrhs, cudaStream_t s) {
     }
   }
   (void)saved;
+  M.settled = was_settled;
   counters().launches += 6 * ncand;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -451,7 +515,8 @@ int autotune_spmv(DBsr<VT>& M, int nrhs, cudaStream_t s) {
 // text form of the cache: "nnzb nbr nbc br bc value_bytes nrhs code" per line
 // (value_bytes + 100 for matrices with the padded 16-byte copy)
 static bool valid_code(int c) {
-  return (c >= 1 && c <= 16) || (c >= 101 && c <= 116) || (c >= 301 && c <= 316);
+  return (c >= 1 && c <= 16) || (c >= 101 && c <= 116) || (c >= 301 && c <= 316) ||
+         (c >= 401 && c <= 416);
 }
 
 void tune_save(const char* path) {
@@ -515,15 +580,17 @@ __global__ void __launch_bounds__(256) k_block_op(int nv, int np, DBsr<double> A
   double acc[NRHS];
 #pragma unroll
   for (int h = 0; h < NRHS; ++h) acc[h] = 0.0;
-  if (!active) {
-  } else if (o < nrow_v) {
-    const int i = (int)(o / 3), r = (int)(o - 3LL * i);
-    scalar_row_accum<3, NRHS, G>(A.rp, A.col, A.val, xv, 3, i, r, lane, acc);
-    scalar_row_accum<1, NRHS, G>(B.rp, B.col, B.val, xp, 3, i, r, lane, acc);
-  } else {
-    const int i = (int)(o - nrow_v);
-    scalar_row_accum<3, NRHS, G>(C.rp, C.col, C.val, xv, 1, i, 0, lane, acc);
-    scalar_row_accum<1, NRHS, G>(D.rp, D.col, D.val, xp, 1, i, 0, lane, acc);
+  const bool vrow = active && o < nrow_v, prow = active && o >= nrow_v;
+  const int iv = vrow ? (int)(o / 3) : 0, r = vrow ? (int)(o - 3LL * iv) : 0;
+  const int ip = prow ? (int)(o - nrow_v) : 0;
+  // the rows of a warp are all of one kind but in the warp where they meet
+  if (__any_sync(0xffffffffu, vrow)) {
+    scalar_row_accum<3, 3, NRHS, G>(A.rp, A.col, A.val, xv, vrow, iv, r, lane, acc);
+    scalar_row_accum<3, 1, NRHS, G>(B.rp, B.col, B.val, xp, vrow, iv, r, lane, acc);
+  }
+  if (__any_sync(0xffffffffu, prow)) {
+    scalar_row_accum<1, 3, NRHS, G>(C.rp, C.col, C.val, xv, prow, ip, 0, lane, acc);
+    scalar_row_accum<1, 1, NRHS, G>(D.rp, D.col, D.val, xp, prow, ip, 0, lane, acc);
   }
 #pragma unroll
   for (int h = 0; h < NRHS; ++h)
@@ -547,10 +614,9 @@ __global__ void __launch_bounds__(256) k_schur_combine(int np, DBsr<T> C, DBsr<T
   T ac[NRHS], ad[NRHS];
 #pragma unroll
   for (int h = 0; h < NRHS; ++h) ac[h] = ad[h] = (T)0;
-  if (active) {
-    scalar_row_accum<3, NRHS, G>(C.rp, C.col, C.val, xt, 1, (int)o, 0, lane, ac);
-    scalar_row_accum<1, NRHS, G>(D.rp, D.col, D.val, xp, 1, (int)o, 0, lane, ad);
-  }
+  const int row = active ? (int)o : 0;
+  scalar_row_accum<1, 3, NRHS, G>(C.rp, C.col, C.val, xt, active, row, 0, lane, ac);
+  scalar_row_accum<1, 1, NRHS, G>(D.rp, D.col, D.val, xp, active, row, 0, lane, ad);
 #pragma unroll
   for (int h = 0; h < NRHS; ++h)
 #pragma unroll
