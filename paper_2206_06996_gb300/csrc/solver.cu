@@ -135,6 +135,9 @@ static DBsr<float> to_float_copy(const DBsr<double>& M, DeviceArena& a, cudaStre
   F.col = M.col;
   F.val = a.alloc<float>(M.nnzb * M.br * M.bc + 1);
   F.g = 0;
+  F.lrow = M.lrow;
+  F.nlong = M.nlong;
+  F.lthr = M.lthr;
   slab_to_float(M.val, F.val, M.nnzb * M.br * M.bc, s);
   return F;
 }
@@ -272,6 +275,21 @@ struct Hierarchy {
       lv.push_back(L);
       break;
     }
+    // long rows of the levels' operators and restrictions (before the smoother
+    // data, whose products a numeric re-set-up runs in the same way)
+    {
+      LongRows lr(ar, s);
+      std::vector<int> ia(lv.size(), -1), ir(lv.size(), -1);
+      for (size_t l = 0; l + 1 < lv.size(); ++l) {
+        if (!lv[l].A.lrow) ia[l] = lr.add(lv[l].A.nbr, lv[l].A.nnzb, lv[l].A.rp);
+        ir[l] = lr.add(lv[l].R.nbr, lv[l].R.nnzb, lv[l].R.rp);
+      }
+      lr.read();
+      for (size_t l = 0; l + 1 < lv.size(); ++l) {
+        if (ia[l] >= 0) lr.set(ia[l], lv[l].A);
+        lr.set(ir[l], lv[l].R);
+      }
+    }
     // coarsest level: dense inverse
     Level& C = lv.back();
     nc = (int)C.n;
@@ -345,24 +363,6 @@ struct Hierarchy {
     if (f32) {
       cinvf = ar.alloc<float>((size_t)nc * nc + 1);
       cast_d2f(cinv, cinvf, (long long)nc * nc, s);
-    }
-    // long rows of the levels' operators and restrictions
-    {
-      LongRows lr(ar, s);
-      std::vector<int> ia(lv.size(), -1), ir(lv.size(), -1);
-      for (size_t l = 0; l + 1 < lv.size(); ++l) {
-        if (!lv[l].A.lrow) ia[l] = lr.add(lv[l].A.nbr, lv[l].A.nnzb, lv[l].A.rp);
-        ir[l] = lr.add(lv[l].R.nbr, lv[l].R.nnzb, lv[l].R.rp);
-      }
-      lr.read();
-      for (size_t l = 0; l + 1 < lv.size(); ++l) {
-        if (ia[l] >= 0) lr.set(ia[l], lv[l].A);
-        lv[l].Af.lrow = lv[l].A.lrow;
-        lv[l].Af.nlong = lv[l].A.nlong;
-        lv[l].Af.lthr = lv[l].A.lthr;
-        lr.set(ir[l], lv[l].R);
-        lr.set(ir[l], lv[l].Rf);
-      }
     }
     // lane-group widths of the products on the two finest levels
     if (o.autotune) {
