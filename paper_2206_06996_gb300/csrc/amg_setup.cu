@@ -14,6 +14,8 @@
 //                  entry in a fixed order (results do not depend on
 //                  scheduling);
 //  coarsest level  dense Gauss-Jordan inverse with partial pivoting.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 
@@ -169,6 +171,10 @@ void power_start_unit(double* v, long long n, const Reducer& red, double* nrm, c
   counters().launches += 2;
 }
 
+// w = -D^{-1} A v is one product (the sign alternates, the norms are those of
+// the power iteration); the vector is normalised every fifth step, which
+// bounds its growth at lambda^5, and before the last step, whose norm is the
+// estimate.  Normalising every step cost six launches a step instead of one.
 double power_lambda(const DBsr<double>& A, const double* dinv, int iters, cudaStream_t s) {
   const long long n = (long long)A.nbr * A.br;
   if (n == 0) return 0.0;
@@ -176,24 +182,29 @@ double power_lambda(const DBsr<double>& A, const double* dinv, int iters, cudaSt
   Reducer red = make_reducer(tmp);
   double* v = tmp.alloc<double>(n);
   double* w = tmp.alloc<double>(n);
+  double* zero = tmp.alloc<double>(n);
   double* nrm = tmp.alloc<double>(2);
-  k_power_start<<<ceil_div(n, 256), 256, 0, s>>>(v, n);
-  SCR_LAUNCH();
-  norm2<double>(v, n, nrm, red, s);
-  k_rsqrt_scalar<<<1, 1, 0, s>>>(nrm, nrm + 1);
-  scale_by<double>(v, nrm + 1, v, n, s);
+  fill<double>(zero, 0.0, n, s);
+  power_start_unit(v, n, red, nrm, s);
+  EpiArgs e;
+  e.kind = Epi::ScaledSub;
+  e.z = zero;
+  e.dinv = dinv;
   for (int it = 0; it < iters; ++it) {
-    spmv<double, double>(A, v, w, 1, EpiArgs(), s);
-    diag_scale<double>(w, dinv, w, n, 1, s);
-    norm2<double>(w, n, nrm, red, s);
-    k_rsqrt_scalar<<<1, 1, 0, s>>>(nrm, nrm + 1);
-    scale_by<double>(w, nrm + 1, v, n, s);
+    spmv<double, double>(A, v, w, 1, e, s);
+    std::swap(v, w);
+    if (it + 1 < iters && (it % 5 == 4 || it + 2 == iters)) {
+      norm2<double>(v, n, nrm, red, s);
+      k_rsqrt_scalar<<<1, 1, 0, s>>>(nrm, nrm + 1);
+      SCR_LAUNCH();
+      counters().launches++;
+      scale_by<double>(v, nrm + 1, v, n, s);
+    }
   }
-  SCR_LAUNCH();
+  norm2<double>(v, n, nrm, red, s);
   double h = 0.0;
   SCR_CUDA(cudaMemcpyAsync(&h, nrm, sizeof(double), cudaMemcpyDeviceToHost, s));
   SCR_CUDA(cudaStreamSynchronize(s));
-  counters().launches += 2 + 2 * iters;
   return 1.1 * std::sqrt(h);
 }
 
@@ -1172,116 +1183,215 @@ void to_dense(const DBsr<double>& A, double* dense, cudaStream_t s) {
   counters().launches++;
 }
 
-// Gauss-Jordan with partial pivoting by one thread block; M and Inv
-// column-major n x n; M is destroyed.
-__global__ void __launch_bounds__(1024) k_gauss_jordan(double* __restrict__ M, double* __restrict__ Inv, int n,
-                                                       int* __restrict__ singular) {
-  extern __shared__ double colk[];
-  __shared__ double rv[32];
-  __shared__ int ri[32];
-  __shared__ int piv;
+// Inverse of the dense coarsest operator: Gauss-Jordan with partial pivoting,
+// in place, by one thread-block cluster.  M is column-major n x n; CTA q of
+// the cluster's NC owns the columns c with c % NC = q, in shared memory where
+// they fit (SM), a warp per column.  Step k: the owner of column k finds the
+// pivot row p and publishes the column with rows k and p exchanged (scratch:
+// 2 n doubles, 2 reciprocals, n pivots), a cluster barrier, then every CTA
+// exchanges the rows in its columns, scales row k and subtracts; column k
+// turns into the inverse's column.  The columns come out in the order of the
+// row exchanges and are put back at the end.
+// One CTA on [M | I] was bound by the FP64 pipe of one SM: 2 n^2 multiply-adds
+// per step at 2 a clock.  16 SMs on n^2 take (192 rows) 2.5 ms -> see
+// dense_inverse.
+__device__ __forceinline__ void invert_publish(const double* a, int k, int n, double* f, double* recip, int* piv,
+                                               int* singular, double* rv, int* ri) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  for (long long e = tid; e < (long long)n * n; e += nt) Inv[e] = (e % (n + 1) == 0) ? 1.0 : 0.0;
+  double best = -1.0;
+  int bi = k;
+  for (int r = k + tid; r < n; r += nt) {
+    const double v = fabs(a[r]);
+    if (v > best) {
+      best = v;
+      bi = r;
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+    if (ov > best || (ov == best && oi < bi)) {
+      best = ov;
+      bi = oi;
+    }
+  }
+  if ((tid & 31) == 0) {
+    rv[tid >> 5] = best;
+    ri[tid >> 5] = bi;
+  }
   __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    // pivot: argmax_{r >= k} |M[r, k]|
-    double best = -1.0;
-    int bi = k;
-    for (int r = k + tid; r < n; r += nt) {
-      const double v = fabs(M[r + (long long)k * n]);
-      if (v > best) {
-        best = v;
-        bi = r;
-      }
+  best = -1.0;
+  int p = k;
+  for (int w = 0; w < nt / 32; ++w)
+    if (rv[w] > best || (rv[w] == best && ri[w] < p)) {
+      best = rv[w];
+      p = ri[w];
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ov = __shfl_down_sync(0xffffffffu, best, o);
-      const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-      if (ov > best || (ov == best && oi < bi)) {
-        best = ov;
-        bi = oi;
-      }
-    }
-    if ((tid & 31) == 0) {
-      rv[tid >> 5] = best;
-      ri[tid >> 5] = bi;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      double b = -1.0;
-      int p = k;
-      for (int w = 0; w < nt / 32; ++w)
-        if (rv[w] > b || (rv[w] == b && ri[w] < p)) {
-          b = rv[w];
-          p = ri[w];
-        }
-      piv = p;
-      if (!(b > 0.0)) *singular = 1;
-    }
-    __syncthreads();
-    const int p = piv;
-    if (p != k) {
-      for (int c = tid; c < n; c += nt) {
-        double t = M[k + (long long)c * n];
-        M[k + (long long)c * n] = M[p + (long long)c * n];
-        M[p + (long long)c * n] = t;
-        t = Inv[k + (long long)c * n];
-        Inv[k + (long long)c * n] = Inv[p + (long long)c * n];
-        Inv[p + (long long)c * n] = t;
-      }
-    }
-    __syncthreads();
-    const double d = M[k + (long long)k * n];
-    const double dinv = d != 0.0 ? 1.0 / d : 0.0;
-    __syncthreads();
-    for (int c = tid; c < n; c += nt) {
-      M[k + (long long)c * n] *= dinv;
-      Inv[k + (long long)c * n] *= dinv;
-    }
-    for (int r = tid; r < n; r += nt) colk[r] = M[r + (long long)k * n];
-    __syncthreads();
-    for (long long e = tid; e < (long long)n * n; e += nt) {
-      const int r = (int)(e % n), c = (int)(e / n);
-      if (r == k) continue;
-      const double f = colk[r];
-      if (f != 0.0) {
-        M[e] -= f * M[k + (long long)c * n];
-        Inv[e] -= f * Inv[k + (long long)c * n];
-      }
-    }
-    __syncthreads();
+  for (int r = tid; r < n; r += nt) f[r] = a[r == k ? p : r == p ? k : r];
+  if (tid == 0) {
+    const double d = a[p];
+    *recip = d != 0.0 ? 1.0 / d : 0.0;
+    *piv = p;
+    if (!(best > 0.0)) *singular = 1;
   }
 }
 
+template <bool SM>
+__global__ void __launch_bounds__(512) k_invert(double* M, double* Inv, int n, int* singular, double* scratch) {
+  extern __shared__ double sm[];
+  const cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  const int q = (int)cl.block_rank(), nc = (int)cl.num_blocks();
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  double* fbuf = scratch;            // two published columns
+  double* recip = scratch + 2 * n;   // their pivots' reciprocals
+  int* piv = reinterpret_cast<int*>(scratch + 2 * n + 2);
+  double* f = sm;                    // the published column of this step
+  double* rv = sm + n;               // pivot search
+  int* ri = reinterpret_cast<int*>(rv + nw);
+  int* pos = ri + nw + (nw & 1);     // column order at the end (n)
+  double* cols = rv + nw + (nw + 1) / 2 + (n + 1) / 2;
+  const int ncol = q < n ? (n - q + nc - 1) / nc : 0;
+  auto column = [&](int lc) { return SM ? cols + (long long)lc * n : M + (long long)(q + lc * nc) * n; };
+  if (SM) {
+    for (int lc = warp; lc < ncol; lc += nw)
+      for (int r = lane; r < n; r += 32) cols[(long long)lc * n + r] = M[(long long)(q + lc * nc) * n + r];
+    __syncthreads();
+  }
+  if (q == 0) invert_publish(column(0), 0, n, fbuf, recip, piv, singular, rv, ri);
+  cl.sync();
+  for (int k = 0; k < n; ++k) {
+    const double* fk = fbuf + (long long)(k & 1) * n;
+    for (int r = tid; r < n; r += nt) f[r] = __ldcg(fk + r);
+    const int p = __ldcg(piv + k);
+    const double di = __ldcg(recip + (k & 1));
+    __syncthreads();
+    for (int lc = warp; lc < ncol; lc += nw) {
+      double* a = column(lc);
+      if (q + lc * nc == k) {
+        for (int r = lane; r < n; r += 32) a[r] = r == k ? di : -f[r] * di;
+        continue;
+      }
+      const double t = a[p] * di, ak = a[k];
+      __syncwarp();
+      for (int r = lane; r < n; r += 32) {
+        const double v = r == p ? ak : a[r], g = f[r];
+        a[r] = r == k ? t : g != 0.0 ? v - g * t : v;
+      }
+    }
+    __syncthreads();
+    if (k + 1 < n && (k + 1) % nc == q)
+      invert_publish(column((k + 1) / nc), k + 1, n, fbuf + (long long)((k + 1) & 1) * n, recip + ((k + 1) & 1),
+                     piv + k + 1, singular, rv, ri);
+    cl.sync();
+  }
+  // undo the exchanges on the columns: from[j] = the computed column that is
+  // column j of the inverse
+  int* from = pos;
+  for (int j = tid; j < n; j += nt) from[j] = j;
+  __syncthreads();
+  if (tid == 0)
+    for (int k = n - 1; k >= 0; --k) {
+      const int p = __ldcg(piv + k), t = from[k];
+      from[k] = from[p];
+      from[p] = t;
+    }
+  __syncthreads();
+  for (int j = warp; j < n; j += nw) {
+    const int c = from[j];
+    if (c % nc != q) continue;
+    const double* a = column(c / nc);
+    for (int r = lane; r < n; r += 32) Inv[(long long)j * n + r] = a[r];
+  }
+}
+
+// 16 CTAs of 512 threads (8 where the device places no cluster of 16).
+// Measured (us): see profiles of the set-up; shared memory holds the columns
+// up to about 560 rows, beyond that they stay in L2.
 void dense_inverse(double* M, double* inv, int n, int* singular, cudaStream_t s) {
   if (n == 0) return;
-  k_gauss_jordan<<<1, 1024, sizeof(double) * n, s>>>(M, inv, n, singular);
-  SCR_LAUNCH();
-  counters().launches++;
+  constexpr int kThreads = 512, kWarps = kThreads / 32;
+  const size_t head = sizeof(double) * (n + kWarps + (kWarps + 1) / 2 + (n + 1) / 2 + 2);
+  for (int nc : {16, 8}) {
+    const size_t cols = sizeof(double) * ((n + nc - 1) / nc) * (size_t)n;
+    const bool fits = head + cols <= 200 * 1024;
+    const size_t bytes = fits ? head + cols : head;
+    auto* kern = fits ? k_invert<true> : k_invert<false>;
+    SCR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    if (nc > 8) SCR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nc);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = bytes;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = nc;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (nc > 8) {
+      int most = 0;
+      if (cudaOccupancyMaxActiveClusters(&most, kern, &cfg) != cudaSuccess || most < 1) {
+        cudaGetLastError();
+        continue;
+      }
+    }
+    DeviceArena tmp(s);
+    double* scratch = tmp.alloc<double>(2 * (size_t)n + 2 + (n + 1) / 2 + 1);
+    SCR_CUDA(cudaLaunchKernelEx(&cfg, kern, M, inv, n, singular, scratch));
+    counters().launches++;
+    return;
+  }
+}
+
+// x = inv b for the coarsest level: 32 rows per CTA, the lanes along a column
+// of inv (coalesced), the columns dealt to the CTA's warps and their sums
+// added in shared memory in warp order.  One thread per row was a chain of n
+// dependent multiply-adds: FP64, 192 rows, 26 us.
+template <int NRHS, typename T>
+__global__ void __launch_bounds__(512) k_dense_apply(const T* __restrict__ inv, const T* b, T* __restrict__ x, int n) {
+  __shared__ T part[16][32 * NRHS + 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane;
+  T acc[NRHS];
+#pragma unroll
+  for (int h = 0; h < NRHS; ++h) acc[h] = (T)0;
+  if (i < n) {
+#pragma unroll 4
+    for (int j = warp; j < n; j += 16) {
+      const T a = inv[i + (long long)j * n];
+#pragma unroll
+      for (int h = 0; h < NRHS; ++h) acc[h] = fma(a, b[(long long)j * NRHS + h], acc[h]);
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < NRHS; ++h) part[warp][lane * NRHS + h] = acc[h];
+  __syncthreads();
+  for (int o = threadIdx.x; o < 32 * NRHS; o += 512) {
+    T v = (T)0;
+#pragma unroll
+    for (int w = 0; w < 16; ++w) v += part[w][o];
+    const long long g = (long long)blockIdx.x * 32 * NRHS + o;
+    if (g < (long long)n * NRHS) x[g] = v;
+  }
 }
 
 template <typename T>
-__global__ void k_dense_apply(const T* __restrict__ inv, const T* __restrict__ b, T* __restrict__ x, int n,
-                              int nrhs) {
-  const int o = blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= n * nrhs) return;
-  const int i = o / nrhs, h = o - i * nrhs;
-  T acc = 0;
-  for (int j = 0; j < n; ++j) acc = fma(inv[i + (long long)j * n], b[(long long)j * nrhs + h], acc);
-  x[o] = acc;
-}
-
-void dense_apply(const double* inv, const double* b, double* x, int n, int nrhs, cudaStream_t s) {
+static void dense_apply_t(const T* inv, const T* b, T* x, int n, int nrhs, cudaStream_t s) {
   if (n == 0) return;
-  k_dense_apply<double><<<ceil_div((long long)n * nrhs, 128), 128, 0, s>>>(inv, b, x, n, nrhs);
+  const int grid = ceil_div(n, 32);
+  if (nrhs == 1) k_dense_apply<1, T><<<grid, 512, 0, s>>>(inv, b, x, n);
+  else if (nrhs == 3) k_dense_apply<3, T><<<grid, 512, 0, s>>>(inv, b, x, n);
+  else if (nrhs == 8) k_dense_apply<8, T><<<grid, 512, 0, s>>>(inv, b, x, n);
+  else throw CudaError{cudaErrorInvalidValue, "dense_apply: unsupported number of right-hand sides"};
   SCR_LAUNCH();
   counters().launches++;
+}
+void dense_apply(const double* inv, const double* b, double* x, int n, int nrhs, cudaStream_t s) {
+  dense_apply_t<double>(inv, b, x, n, nrhs, s);
 }
 void dense_apply_f(const float* inv, const float* b, float* x, int n, int nrhs, cudaStream_t s) {
-  if (n == 0) return;
-  k_dense_apply<float><<<ceil_div((long long)n * nrhs, 128), 128, 0, s>>>(inv, b, x, n, nrhs);
-  SCR_LAUNCH();
-  counters().launches++;
+  dense_apply_t<float>(inv, b, x, n, nrhs, s);
 }
 
 }  // namespace scr

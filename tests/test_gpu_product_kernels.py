@@ -66,3 +66,20 @@ def test_vcycle_with_long_rows_matches_oracle(code):
         x = sol.amg_apply(pkg.SCR_HIER_A, _dev(b)).cpu().numpy()
     ref = amg.vcycle(amg.hierarchy_from_matrices(As, Ps, 3, 1, 1, "cheb", 3), b)
     assert np.linalg.norm(x - ref) <= 1e-11 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("preset,which,bs", [("tube_tiny", pkg.SCR_HIER_A, 3), ("tube_mini", pkg.SCR_HIER_SHAT, 1),
+                                             ("tube_mini", pkg.SCR_HIER_A, 3)])
+def test_dense_coarsest_solve_inverts_the_operator(preset, which, bs):
+    """A hierarchy of one level is the dense inverse alone: 81 and 949 rows in
+    one cluster's shared memory or in L2, 2,379 rows in L2; x = A^{-1} b has
+    the residual of an explicit inverse, at most 8 n eps cond(A) |b|."""
+    s = F.tube_system(preset)
+    with pkg.BlockSolver(amg_max_levels=1) as sol:
+        sol.setup(s.A, s.B, s.C, s.D)
+        A = to_csr(sol.export(which, 0, pkg.SCR_EXPORT_OPERATOR)).toarray()
+        n = A.shape[0]
+        b = np.random.default_rng(n).standard_normal(n)
+        x = sol.amg_apply(which, _dev(b)).cpu().numpy()
+    tol = 8 * n * np.finfo(float).eps * np.linalg.cond(A)
+    assert np.linalg.norm(A @ x - b) <= tol * np.linalg.norm(b)
