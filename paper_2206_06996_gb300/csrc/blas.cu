@@ -15,6 +15,8 @@ Reducer make_reducer(DeviceArena& a) {
   Reducer r;
   r.nblk = std::min(2 * sm_count(), 1024);
   r.partial = a.alloc<double>((size_t)r.nblk * kMaxBasis);
+  r.ticket = a.alloc<unsigned>(1);
+  SCR_CUDA(cudaMemsetAsync(r.ticket, 0, sizeof(unsigned), a.stream()));
   return r;
 }
 
@@ -47,24 +49,6 @@ __global__ void k_scale_by(const T* __restrict__ x, const double* __restrict__ s
   long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x, st = (long long)gridDim.x * blockDim.x;
   for (; i < n; i += st) y[i] = a * x[i];
 }
-// y = x (times *sc when sc is given), with x and/or y a column of a basis
-// whose index is read on the device: column (*xj) of X, column (*yj + yoff)
-// of Y (stride ld); a null index pointer names the vector itself
-template <typename T>
-__global__ void k_col_copy(const T* __restrict__ X, const int* __restrict__ xj, T* __restrict__ Y,
-                           const int* __restrict__ yj, int yoff, long long ld, const double* __restrict__ sc,
-                           long long n) {
-  const T* x = xj ? X + (long long)*xj * ld : X;
-  T* y = yj ? Y + (long long)(*yj + yoff) * ld : Y;
-  long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x, st = (long long)gridDim.x * blockDim.x;
-  if (sc) {
-    const T a = (T)*sc;
-    for (; i < n; i += st) y[i] = a * x[i];
-  } else {
-    for (; i < n; i += st) y[i] = x[i];
-  }
-}
-
 static int grid_for(long long n) {
   return (int)std::max<long long>(1, std::min<long long>(ceil_div(n, 256), 8LL * sm_count()));
 }
@@ -255,18 +239,31 @@ void scale_by(const T* x, const double* sc, T* y, long long n, cudaStream_t s) {
 
 template void scale_by<double>(const double*, const double*, double*, long long, cudaStream_t);
 
+// y = column *yj + yoff of Y (Y itself without yj) = a x with a = *sc, and z = y
 template <typename T>
-void col_copy(const T* X, const int* xj, T* Y, const int* yj, int yoff, long long ld, const double* sc, long long n,
-              cudaStream_t s) {
+__global__ void k_scale_two(const T* __restrict__ x, const double* __restrict__ sc, T* __restrict__ Y,
+                            const int* __restrict__ yj, int yoff, long long ld, T* __restrict__ z, long long n) {
+  T* y = yj ? Y + (long long)(*yj + yoff) * ld : Y;
+  const T a = (T)*sc;
+  long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x, st = (long long)gridDim.x * blockDim.x;
+  for (; i < n; i += st) {
+    const T v = a * x[i];
+    y[i] = v;
+    z[i] = v;
+  }
+}
+template <typename T>
+void scale_two(const T* x, const double* sc, T* Y, const int* yj, int yoff, long long ld, T* z, long long n,
+               cudaStream_t s) {
   if (n <= 0) return;
-  k_col_copy<T><<<grid_for(n), 256, 0, s>>>(X, xj, Y, yj, yoff, ld, sc, n);
+  k_scale_two<T><<<grid_for(n), 256, 0, s>>>(x, sc, Y, yj, yoff, ld, z, n);
   SCR_LAUNCH();
   counters().launches++;
 }
-template void col_copy<double>(const double*, const int*, double*, const int*, int, long long, const double*,
-                               long long, cudaStream_t);
-template void col_copy<float>(const float*, const int*, float*, const int*, int, long long, const double*,
-                              long long, cudaStream_t);
+template void scale_two<double>(const double*, const double*, double*, const int*, int, long long, double*, long long,
+                                cudaStream_t);
+template void scale_two<float>(const float*, const double*, float*, const int*, int, long long, float*, long long,
+                               cudaStream_t);
 
 template <typename T>
 __global__ void k_axpby_t(T a, const T* __restrict__ x, T b, T* __restrict__ y, long long n) {
@@ -358,34 +355,170 @@ __device__ __forceinline__ void store_partials_t(T (&acc)[KMAX], int k, double* 
   block_store_partials<KMAX>(d, k, partial);
 }
 
-// Counts: k, or (*kp + koff) when kp is given (a count kept on the device
-// by a loop recorded in a CUDA graph; KMAX bounds it either way).
+// ------------------------------------------------------------ reduction tails
+// Arnoldi scalars of column j by one warp: the lanes load column j of H (the
+// two Gram-Schmidt passes' coefficients) and the previous rotations into
+// shared memory in parallel, lane 0 applies the rotations and the new one
+// there, the lanes write the column back.
+__device__ __forceinline__ void arnoldi_column(ArnoldiState* st, int j, double* host_rel) {
+  constexpr int ldh = kMaxBasis + 1;
+  __shared__ double h[kMaxBasis + 2], rc[kMaxBasis], rs[kMaxBasis];
+  const int t = threadIdx.x & 31;
+  double* Hj = st->H + (long long)j * ldh;
+  for (int i = t; i <= j; i += 32) h[i] = st->h1[i] + st->h2[i];
+  for (int i = t; i < j; i += 32) {
+    rc[i] = st->cs[i];
+    rs[i] = st->sn[i];
+  }
+  __syncwarp();
+  if (t == 0) {
+    const double hn = sqrt(fmax(st->nrm2, 0.0));
+    st->inv_hnext = hn > 1e-300 ? 1.0 / hn : 0.0;
+    h[j + 1] = hn;
+    // previous rotations
+    for (int i = 0; i < j; ++i) {
+      const double v = rc[i] * h[i] + rs[i] * h[i + 1];
+      h[i + 1] = -rs[i] * h[i] + rc[i] * h[i + 1];
+      h[i] = v;
+    }
+    const double a = h[j], c = h[j + 1];
+    const double d = hypot(a, c);
+    double cs = 1.0, sn = 0.0;
+    if (d != 0.0) {
+      cs = a / d;
+      sn = c / d;
+    }
+    st->cs[j] = cs;
+    st->sn[j] = sn;
+    h[j] = d;
+    h[j + 1] = 0.0;
+    const double gj = st->g[j];
+    st->g[j + 1] = -sn * gj;
+    st->g[j] = cs * gj;
+    st->rel = fabs(st->g[j + 1]) / st->bnorm;
+    // happy breakdown: the new direction vanished relative to the column
+    st->breakdown = (hn <= 1e-300 || d == 0.0) ? 1 : 0;
+    if (host_rel) {
+      host_rel[0] = st->rel;
+      host_rel[1] = (double)st->breakdown;
+    }
+  }
+  __syncwarp();
+  for (int i = t; i <= j + 1; i += 32) Hj[i] = h[i];
+}
+
+// a device loop's step: counts it and sets the loop's condition
+__device__ __forceinline__ void loop_next(const ArnoldiState* st, const LoopStep& c) {
+  KrylovLoop* L = c.L;
+  const int j = L->j + 1, it = L->iters + 1;
+  L->j = j;
+  L->iters = it;
+  L->tot_iters++;
+  const double r = st->rel;
+  L->rel = r;
+  const bool fin = isfinite(r);
+  if (!fin) {  // the host loop returns here without the update: a zero count skips it
+    L->nonfinite = 1;
+    L->j = 0;
+  }
+  const bool go = fin && !(r <= c.tol) && st->breakdown == 0 && j < c.m && it < c.maxit;
+  cudaGraphSetConditional(c.handle, go ? 1u : 0u);
+}
+
+__device__ __forceinline__ void cg_scalar(CgState* st, int mode, double* host_rel) {
+  switch (mode) {
+    case Tail::CgStart:  // bnorm2 in rr
+      st->bnorm2 = st->rr;
+      st->rel = st->rr > 0 ? 1.0 : 0.0;
+      if (host_rel) host_rel[0] = st->rel, host_rel[1] = st->bnorm2;
+      break;
+    case Tail::CgAlpha:  // alpha = rz / pq
+      st->alpha = st->pq != 0.0 ? st->rz / st->pq : 0.0;
+      break;
+    case Tail::CgRel:  // residual estimate
+      st->rel = st->bnorm2 > 0 ? sqrt(st->rr / st->bnorm2) : 0.0;
+      if (host_rel) host_rel[0] = st->rel;
+      break;
+    case Tail::CgFirst:  // first rz
+      st->rz = st->rz_new;
+      break;
+    case Tail::CgBeta:  // beta = rz_new / rz
+      st->beta = st->rz != 0.0 ? st->rz_new / st->rz : 0.0;
+      st->rz = st->rz_new;
+      break;
+    default:
+      break;
+  }
+}
+
+// The end of a reduction: the CTA that finishes last adds the CTAs' partial
+// sums in CTA order (a warp per sum, the lanes a stride of 32 each, so the
+// result does not depend on which CTA that is) and runs what follows from the
+// sums.  A kernel of its own for this cost a launch and a pass of one CTA per
+// reduction: 3.5 us, three times per Arnoldi step.
+__device__ __forceinline__ void reduce_tail(const double* partial, int k, double* out, unsigned* ticket,
+                                            const Tail& t) {
+  __shared__ bool last;
+  __threadfence();  // this thread's partial sum is visible before the ticket counts it
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int j = wid; j < k; j += nw) {
+    double v = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) v += __ldcg(partial + (long long)b * kMaxBasis + j);
+    v = warp_sum(v);
+    if (lane == 0) out[j] = v;
+  }
+  if (threadIdx.x == 0) *ticket = 0;  // for the next reduction on this stream
+  if (t.what == Tail::None) return;
+  __syncthreads();
+  if (t.what == Tail::Arnoldi) {
+    if (wid == 0) {
+      arnoldi_column(t.st, t.jp ? *t.jp : t.j, t.host_rel);
+      __syncwarp();
+      if (lane == 0 && t.loop.L) loop_next(t.st, t.loop);
+    }
+  } else if (threadIdx.x == 0) {
+    cg_scalar(t.cg, t.what, t.host_rel);
+  }
+}
+
+// where a reduction's sums go
+struct Sink {
+  double* partial;
+  double* out;
+  unsigned* ticket;
+  Tail tail;
+};
+
 template <int KMAX, typename T>
 __global__ void __launch_bounds__(kRedThreads) k_multidot(const T* __restrict__ V, long long ld, int k,
                                                          const T* __restrict__ w, long long n,
-                                                         double* __restrict__ partial, const int* __restrict__ kp,
-                                                         int koff) {
-  if (kp) k = *kp + koff;
+                                                         const T* __restrict__ keep, T* __restrict__ kept,
+                                                         Sink sink) {
   T acc[KMAX];
 #pragma unroll
   for (int j = 0; j < KMAX; ++j) acc[j] = (T)0;
   const long long st = (long long)gridDim.x * blockDim.x;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += st) {
     const T wi = w[i];
+    if (keep) kept[i] = keep[i];
 #pragma unroll
     for (int j = 0; j < KMAX; ++j)
       if (j < k) acc[j] = fma(V[j * ld + i], wi, acc[j]);
   }
-  store_partials_t<KMAX, T>(acc, k, partial);
+  store_partials_t<KMAX, T>(acc, k, sink.partial);
+  reduce_tail(sink.partial, k, sink.out, sink.ticket, sink.tail);
 }
 
 // w -= V h; partial sums of V_j . w (new)
 template <int KMAX, typename T>
 __global__ void __launch_bounds__(kRedThreads) k_cgs_update_dot(const T* __restrict__ V, long long ld, int k,
                                                                const double* __restrict__ h, T* __restrict__ w,
-                                                               long long n, double* __restrict__ partial,
-                                                               const int* __restrict__ kp, int koff) {
-  if (kp) k = *kp + koff;
+                                                               long long n, Sink sink) {
   T hj[KMAX], acc[KMAX];
 #pragma unroll
   for (int j = 0; j < KMAX; ++j) {
@@ -403,16 +536,15 @@ __global__ void __launch_bounds__(kRedThreads) k_cgs_update_dot(const T* __restr
     for (int j = 0; j < KMAX; ++j)
       if (j < k) acc[j] = fma(V[j * ld + i], wi, acc[j]);
   }
-  store_partials_t<KMAX, T>(acc, k, partial);
+  store_partials_t<KMAX, T>(acc, k, sink.partial);
+  reduce_tail(sink.partial, k, sink.out, sink.ticket, sink.tail);
 }
 
 // w -= V h; partial sum of w . w
 template <int KMAX, typename T>
 __global__ void __launch_bounds__(kRedThreads) k_cgs_update_norm(const T* __restrict__ V, long long ld, int k,
                                                                 const double* __restrict__ h, T* __restrict__ w,
-                                                                long long n, double* __restrict__ partial,
-                                                                const int* __restrict__ kp, int koff) {
-  if (kp) k = *kp + koff;
+                                                                long long n, Sink sink) {
   T hj[KMAX];
 #pragma unroll
   for (int j = 0; j < KMAX; ++j) hj[j] = j < k ? (T)h[j] : (T)0;
@@ -426,7 +558,8 @@ __global__ void __launch_bounds__(kRedThreads) k_cgs_update_norm(const T* __rest
     w[i] = wi;
     acc[0] = fma(wi, wi, acc[0]);
   }
-  store_partials_t<1, T>(acc, 1, partial);
+  store_partials_t<1, T>(acc, 1, sink.partial);
+  reduce_tail(sink.partial, 1, sink.out, sink.ticket, sink.tail);
 }
 
 // Device-count variants (loops recorded in a CUDA graph): the count k is
@@ -482,9 +615,16 @@ template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_multidot_dev(const T* __restrict__ V, long long ld,
                                                              const int* __restrict__ kp, int koff,
                                                              const T* __restrict__ w, long long n,
-                                                             double* __restrict__ partial) {
+                                                             const T* __restrict__ keep, T* __restrict__ kept,
+                                                             Sink sink) {
   const int k = *kp + koff;
-  for (int c0 = 0; c0 < k; c0 += kDotTile) chunk_dots<T>(V, ld, c0, k, w, n, partial);
+  if (keep) {  // column k - 1 of kept = keep, on the way
+    T* to = kept + (long long)(k - 1) * ld;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+      to[i] = keep[i];
+  }
+  for (int c0 = 0; c0 < k; c0 += kDotTile) chunk_dots<T>(V, ld, c0, k, w, n, sink.partial);
+  reduce_tail(sink.partial, k, sink.out, sink.ticket, sink.tail);
 }
 
 // w -= V h (columns in increasing order), then the dots of the updated w
@@ -493,7 +633,7 @@ template <bool NORM, typename T>
 __global__ void __launch_bounds__(kRedThreads) k_cgs_update_dev(const T* __restrict__ V, long long ld,
                                                                const int* __restrict__ kp, int koff,
                                                                const double* __restrict__ h, T* __restrict__ w,
-                                                               long long n, double* __restrict__ partial) {
+                                                               long long n, Sink sink) {
   __shared__ T hs[kMaxBasis + 1];
   const int k = *kp + koff;
   for (int j = threadIdx.x; j < k; j += blockDim.x) hs[j] = (T)h[j];
@@ -516,40 +656,34 @@ __global__ void __launch_bounds__(kRedThreads) k_cgs_update_dev(const T* __restr
     }
   }
   if constexpr (NORM) {
-    store_chunk_partials<T>(acc, 0, 1, partial);
+    store_chunk_partials<T>(acc, 0, 1, sink.partial);
   } else {
-    store_chunk_partials<T>(acc, 0, k, partial);
-    for (int c0 = kDotTile; c0 < k; c0 += kDotTile) chunk_dots<T>(V, ld, c0, k, w, n, partial);
+    store_chunk_partials<T>(acc, 0, k, sink.partial);
+    for (int c0 = kDotTile; c0 < k; c0 += kDotTile) chunk_dots<T>(V, ld, c0, k, w, n, sink.partial);
   }
+  reduce_tail(sink.partial, NORM ? 1 : k, sink.out, sink.ticket, sink.tail);
 }
 
-// out[j] = sum_b partial[b][j], fixed order
-__global__ void k_reduce_partials(const double* __restrict__ partial, int nblk, int k, double* __restrict__ out,
-                                  const int* __restrict__ kp, int koff) {
-  if (kp) k = *kp + koff;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int j = wid; j < k; j += nw) {
-    double v = 0.0;
-    for (int b = lane; b < nblk; b += 32) v += partial[(long long)b * kMaxBasis + j];
-    v = warp_sum(v);
-    if (lane == 0) out[j] = v;
-  }
+// CTAs of a reduction over n entries: one entry per thread at least
+static int red_grid(const Reducer& r, long long n) {
+  return (int)std::max<long long>(1, std::min<long long>(r.nblk, ceil_div(n, kRedThreads)));
 }
+static Sink sink_of(const Reducer& r, double* out, const Tail& t) { return Sink{r.partial, out, r.ticket, t}; }
 
 template <int KMAX, typename T>
 static void launch_multidot(const T* V, long long ld, int k, const T* w, long long n, const Reducer& r,
-                            cudaStream_t s, const int* kp, int koff) {
-  k_multidot<KMAX, T><<<r.nblk, kRedThreads, 0, s>>>(V, ld, k, w, n, r.partial, kp, koff);
+                            cudaStream_t s, const T* keep, T* kept, const Sink& o) {
+  k_multidot<KMAX, T><<<red_grid(r, n), kRedThreads, 0, s>>>(V, ld, k, w, n, keep, kept, o);
 }
 template <int KMAX, typename T>
 static void launch_cgs_dot(const T* V, long long ld, int k, const double* h, T* w, long long n, const Reducer& r,
-                           cudaStream_t s, const int* kp, int koff) {
-  k_cgs_update_dot<KMAX, T><<<r.nblk, kRedThreads, 0, s>>>(V, ld, k, h, w, n, r.partial, kp, koff);
+                           cudaStream_t s, const Sink& o) {
+  k_cgs_update_dot<KMAX, T><<<red_grid(r, n), kRedThreads, 0, s>>>(V, ld, k, h, w, n, o);
 }
 template <int KMAX, typename T>
 static void launch_cgs_norm(const T* V, long long ld, int k, const double* h, T* w, long long n, const Reducer& r,
-                            cudaStream_t s, const int* kp, int koff) {
-  k_cgs_update_norm<KMAX, T><<<r.nblk, kRedThreads, 0, s>>>(V, ld, k, h, w, n, r.partial, kp, koff);
+                            cudaStream_t s, const Sink& o) {
+  k_cgs_update_norm<KMAX, T><<<red_grid(r, n), kRedThreads, 0, s>>>(V, ld, k, h, w, n, o);
 }
 
 #define SCR_KDISPATCH(FN, T, k, ...)                \
@@ -562,117 +696,55 @@ static void launch_cgs_norm(const T* V, long long ld, int k, const double* h, T*
     else FN<kMaxBasis, T>(__VA_ARGS__);             \
   } while (0)
 
-static void reduce(const Reducer& r, int k, double* out, cudaStream_t s, const int* kp = nullptr, int koff = 0) {
-  k_reduce_partials<<<1, 256, 0, s>>>(r.partial, r.nblk, k, out, kp, koff);
-  SCR_LAUNCH();
-  counters().launches += 2;
-}
-
 template <typename T>
-void norm2(const T* x, long long n, double* out, const Reducer& r, cudaStream_t s) {
-  launch_multidot<1, T>(x, 0, 1, x, n, r, s, nullptr, 0);
+void norm2(const T* x, long long n, double* out, const Reducer& r, cudaStream_t s, const Tail& t) {
+  launch_multidot<1, T>(x, 0, 1, x, n, r, s, nullptr, nullptr, sink_of(r, out, t));
   SCR_LAUNCH();
-  reduce(r, 1, out, s);
+  counters().launches++;
 }
 
 template <typename T>
 void multidot(const T* V, long long ld, int k, const T* w, long long n, double* out, const Reducer& r,
-              cudaStream_t s, const int* kp, int koff) {
-  if (kp) k_multidot_dev<T><<<r.nblk, kRedThreads, 0, s>>>(V, ld, kp, koff, w, n, r.partial);
-  else SCR_KDISPATCH(launch_multidot, T, k, V, ld, k, w, n, r, s, kp, koff);
+              cudaStream_t s, const int* kp, int koff, const Tail& t, const T* keep, T* kept) {
+  const Sink o = sink_of(r, out, t);
+  if (kp) k_multidot_dev<T><<<red_grid(r, n), kRedThreads, 0, s>>>(V, ld, kp, koff, w, n, keep, kept, o);
+  else SCR_KDISPATCH(launch_multidot, T, k, V, ld, k, w, n, r, s, keep, kept ? kept + (long long)(k - 1) * ld : kept, o);
   SCR_LAUNCH();
-  reduce(r, k, out, s, kp, koff);
+  counters().launches++;
 }
 
 template <typename T>
 void cgs_update_dot(const T* V, long long ld, int k, const double* h, T* w, long long n, double* out,
                     const Reducer& r, cudaStream_t s, const int* kp, int koff) {
-  if (kp) k_cgs_update_dev<false, T><<<r.nblk, kRedThreads, 0, s>>>(V, ld, kp, koff, h, w, n, r.partial);
-  else SCR_KDISPATCH(launch_cgs_dot, T, k, V, ld, k, h, w, n, r, s, kp, koff);
-  SCR_LAUNCH();
-  reduce(r, k, out, s, kp, koff);
-}
-
-template <typename T>
-void cgs_update_norm(const T* V, long long ld, int k, const double* h, T* w, long long n, double* out,
-                     const Reducer& r, cudaStream_t s, const int* kp, int koff) {
-  if (kp) k_cgs_update_dev<true, T><<<r.nblk, kRedThreads, 0, s>>>(V, ld, kp, koff, h, w, n, r.partial);
-  else SCR_KDISPATCH(launch_cgs_norm, T, k, V, ld, k, h, w, n, r, s, kp, koff);
-  SCR_LAUNCH();
-  reduce(r, 1, out, s);
-}
-
-#define SCR_INST_BLAS(T)                                                                                      \
-  template void norm2<T>(const T*, long long, double*, const Reducer&, cudaStream_t);                         \
-  template void multidot<T>(const T*, long long, int, const T*, long long, double*, const Reducer&,           \
-                            cudaStream_t, const int*, int);                                                   \
-  template void cgs_update_dot<T>(const T*, long long, int, const double*, T*, long long, double*,            \
-                                  const Reducer&, cudaStream_t, const int*, int);                             \
-  template void cgs_update_norm<T>(const T*, long long, int, const double*, T*, long long, double*,           \
-                                   const Reducer&, cudaStream_t, const int*, int);
-SCR_INST_BLAS(double)
-SCR_INST_BLAS(float)
-
-// ------------------------------------------------------------ Arnoldi scalars
-// One warp: the lanes load column j of H (the two Gram-Schmidt passes'
-// coefficients) and the previous rotations into shared memory in parallel,
-// lane 0 applies the rotations and the new one there (the same operations
-// in the same order as a single thread on the state), the lanes write the
-// column back.
-__global__ void k_arnoldi_finalize(ArnoldiState* st, int j, double* host_rel, const int* __restrict__ jp) {
-  if (jp) j = *jp;
-  constexpr int ldh = kMaxBasis + 1;
-  __shared__ double h[kMaxBasis + 2], rc[kMaxBasis], rs[kMaxBasis];
-  const int t = threadIdx.x;
-  double* Hj = st->H + (long long)j * ldh;
-  for (int i = t; i <= j; i += 32) h[i] = st->h1[i] + st->h2[i];
-  for (int i = t; i < j; i += 32) {
-    rc[i] = st->cs[i];
-    rs[i] = st->sn[i];
-  }
-  __syncwarp();
-  if (t == 0) {
-    const double hn = sqrt(fmax(st->nrm2, 0.0));
-    h[j + 1] = hn;
-    // previous rotations
-    for (int i = 0; i < j; ++i) {
-      const double v = rc[i] * h[i] + rs[i] * h[i + 1];
-      h[i + 1] = -rs[i] * h[i] + rc[i] * h[i + 1];
-      h[i] = v;
-    }
-    const double a = h[j], c = h[j + 1];
-    const double d = hypot(a, c);
-    double cs = 1.0, sn = 0.0;
-    if (d != 0.0) {
-      cs = a / d;
-      sn = c / d;
-    }
-    st->cs[j] = cs;
-    st->sn[j] = sn;
-    h[j] = d;
-    h[j + 1] = 0.0;
-    const double gj = st->g[j];
-    st->g[j + 1] = -sn * gj;
-    st->g[j] = cs * gj;
-    st->rel = fabs(st->g[j + 1]) / st->bnorm;
-    // happy breakdown: the new direction vanished relative to the column
-    st->breakdown = (hn <= 1e-300 || d == 0.0) ? 1 : 0;
-    st->inv_hnext = hn > 1e-300 ? 1.0 / hn : 0.0;
-    if (host_rel) {
-      host_rel[0] = st->rel;
-      host_rel[1] = (double)st->breakdown;
-    }
-  }
-  __syncwarp();
-  for (int i = t; i <= j + 1; i += 32) Hj[i] = h[i];
-}
-
-void arnoldi_finalize(ArnoldiState* st, int j, double* host_rel, cudaStream_t s, const int* jp) {
-  k_arnoldi_finalize<<<1, 32, 0, s>>>(st, j, host_rel, jp);
+  const Sink o = sink_of(r, out, Tail());
+  if (kp) k_cgs_update_dev<false, T><<<red_grid(r, n), kRedThreads, 0, s>>>(V, ld, kp, koff, h, w, n, o);
+  else SCR_KDISPATCH(launch_cgs_dot, T, k, V, ld, k, h, w, n, r, s, o);
   SCR_LAUNCH();
   counters().launches++;
 }
 
+template <typename T>
+void cgs_update_norm(const T* V, long long ld, int k, const double* h, T* w, long long n, double* out,
+                     const Reducer& r, cudaStream_t s, const int* kp, int koff, const Tail& t) {
+  const Sink o = sink_of(r, out, t);
+  if (kp) k_cgs_update_dev<true, T><<<red_grid(r, n), kRedThreads, 0, s>>>(V, ld, kp, koff, h, w, n, o);
+  else SCR_KDISPATCH(launch_cgs_norm, T, k, V, ld, k, h, w, n, r, s, o);
+  SCR_LAUNCH();
+  counters().launches++;
+}
+
+#define SCR_INST_BLAS(T)                                                                                      \
+  template void norm2<T>(const T*, long long, double*, const Reducer&, cudaStream_t, const Tail&);            \
+  template void multidot<T>(const T*, long long, int, const T*, long long, double*, const Reducer&,           \
+                            cudaStream_t, const int*, int, const Tail&, const T*, T*);                        \
+  template void cgs_update_dot<T>(const T*, long long, int, const double*, T*, long long, double*,            \
+                                  const Reducer&, cudaStream_t, const int*, int);                             \
+  template void cgs_update_norm<T>(const T*, long long, int, const double*, T*, long long, double*,           \
+                                   const Reducer&, cudaStream_t, const int*, int, const Tail&);
+SCR_INST_BLAS(double)
+SCR_INST_BLAS(float)
+
+// ------------------------------------------------------------ Arnoldi scalars
 __global__ void k_arnoldi_start(ArnoldiState* st, int first, double* host_rel) {
   const double beta = sqrt(fmax(st->nrm2, 0.0));
   st->beta = beta;
@@ -743,32 +815,8 @@ template void gmres_update<float>(ArnoldiState*, int, const float*, long long, f
                                   const int*);
 
 // ------------------------------------------------------------ CG
-__global__ void k_cg_scalar(CgState* st, int mode, double* host_rel) {
-  switch (mode) {
-    case 0:  // start: bnorm2 in rr
-      st->bnorm2 = st->rr;
-      st->rel = st->rr > 0 ? 1.0 : 0.0;
-      if (host_rel) host_rel[0] = st->rel, host_rel[1] = st->bnorm2;
-      break;
-    case 1:  // alpha = rz / pq
-      st->alpha = st->pq != 0.0 ? st->rz / st->pq : 0.0;
-      break;
-    case 2:  // residual estimate
-      st->rel = st->bnorm2 > 0 ? sqrt(st->rr / st->bnorm2) : 0.0;
-      if (host_rel) host_rel[0] = st->rel;
-      break;
-    case 3:  // first rz
-      st->rz = st->rz_new;
-      break;
-    case 4:  // beta = rz_new / rz
-      st->beta = st->rz != 0.0 ? st->rz_new / st->rz : 0.0;
-      st->rz = st->rz_new;
-      break;
-  }
-}
-
 __global__ void k_cg_xr(const CgState* __restrict__ st, const double* __restrict__ p, const double* __restrict__ q,
-                        double* __restrict__ x, double* __restrict__ r, long long n, double* __restrict__ partial) {
+                        double* __restrict__ x, double* __restrict__ r, long long n, Sink sink) {
   const double a = st->alpha;
   double acc[1] = {0.0};
   const long long stp = (long long)gridDim.x * blockDim.x;
@@ -778,7 +826,8 @@ __global__ void k_cg_xr(const CgState* __restrict__ st, const double* __restrict
     r[i] = ri;
     acc[0] = fma(ri, ri, acc[0]);
   }
-  block_store_partials<1>(acc, 1, partial);
+  block_store_partials<1>(acc, 1, sink.partial);
+  reduce_tail(sink.partial, 1, sink.out, sink.ticket, sink.tail);
 }
 
 __global__ void k_cg_p(const CgState* __restrict__ st, const double* __restrict__ z, double* __restrict__ p,
@@ -788,33 +837,29 @@ __global__ void k_cg_p(const CgState* __restrict__ st, const double* __restrict_
   for (; i < n; i += stp) p[i] = fma(b, p[i], z[i]);
 }
 
+static Tail cg_tail(Tail::What what, CgState* st, double* host_rel = nullptr) {
+  Tail t;
+  t.what = what;
+  t.cg = st;
+  t.host_rel = host_rel;
+  return t;
+}
 void cg_start(CgState* st, const double* b, long long n, const Reducer& red, double* host_rel, cudaStream_t s) {
-  norm2(b, n, &st->rr, red, s);
-  k_cg_scalar<<<1, 1, 0, s>>>(st, 0, host_rel);
-  SCR_LAUNCH();
-  counters().launches++;
+  norm2(b, n, &st->rr, red, s, cg_tail(Tail::CgStart, st, host_rel));
 }
 void cg_dot_rz(CgState* st, const double* r, const double* z, long long n, const Reducer& red, int first,
                cudaStream_t s) {
-  multidot(r, 0, 1, z, n, &st->rz_new, red, s);
-  k_cg_scalar<<<1, 1, 0, s>>>(st, first ? 3 : 4, nullptr);
-  SCR_LAUNCH();
-  counters().launches++;
+  multidot(r, 0, 1, z, n, &st->rz_new, red, s, nullptr, 0, cg_tail(first ? Tail::CgFirst : Tail::CgBeta, st));
 }
 void cg_alpha(CgState* st, const double* p, const double* q, long long n, const Reducer& red, cudaStream_t s) {
-  multidot(p, 0, 1, q, n, &st->pq, red, s);
-  k_cg_scalar<<<1, 1, 0, s>>>(st, 1, nullptr);
-  SCR_LAUNCH();
-  counters().launches++;
+  multidot(p, 0, 1, q, n, &st->pq, red, s, nullptr, 0, cg_tail(Tail::CgAlpha, st));
 }
 void cg_step_x_r(CgState* st, const double* p, const double* q, double* x, double* r, long long n,
                  const Reducer& red, double* host_rel, cudaStream_t s) {
-  k_cg_xr<<<red.nblk, kRedThreads, 0, s>>>(st, p, q, x, r, n, red.partial);
+  k_cg_xr<<<red_grid(red, n), kRedThreads, 0, s>>>(st, p, q, x, r, n,
+                                                  sink_of(red, &st->rr, cg_tail(Tail::CgRel, st, host_rel)));
   SCR_LAUNCH();
-  reduce(red, 1, &st->rr, s);
-  k_cg_scalar<<<1, 1, 0, s>>>(st, 2, host_rel);
-  SCR_LAUNCH();
-  counters().launches += 2;
+  counters().launches++;
 }
 void cg_update_p(CgState* st, const double* z, double* p, long long n, cudaStream_t s) {
   k_cg_p<<<grid_for(n), 256, 0, s>>>(st, z, p, n);

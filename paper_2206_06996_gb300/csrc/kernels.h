@@ -208,9 +208,47 @@ struct ArnoldiState {           // device-resident Krylov scalars
   double beta, bnorm, rel, inv_hnext, nrm2;
   int breakdown;
 };
-struct Reducer {  // partial-sum scratch for deterministic two-stage reductions
+// Scratch of deterministic reductions: each CTA's partial sums and the count
+// of CTAs that are done (zero between reductions).  Reductions that share one
+// run one after another on a stream.
+struct Reducer {
   double* partial = nullptr;  // [nblk * kMaxBasis]
+  unsigned* ticket = nullptr;
   int nblk = 0;
+};
+// state of a GMRES solve recorded as a device loop (solver.cu)
+struct KrylovLoop {
+  int j;          // Arnoldi step inside the current cycle
+  int iters;      // Arnoldi steps of the current solve
+  int cycles;     // restart cycles of the current solve
+  int nonfinite;  // 1 when an estimate was NaN or infinite
+  double rel;     // last residual estimate
+  // since the last reset (read back once per outer solve for the counters)
+  long long tot_iters, tot_solves, tot_cycles, tot_restarts;
+};
+struct LoopStep {  // the end of a device loop's Arnoldi step (L null: none)
+  KrylovLoop* L = nullptr;
+  cudaGraphConditionalHandle handle = 0;
+  double tol = 0.0;
+  int m = 0, maxit = 0;
+};
+struct CgState {
+  double rz, rz_new, pq, alpha, beta, rr, bnorm2, rel;
+};
+// What the last CTA of a reduction does with the sums.
+// Arnoldi: bookkeeping for column j (or *jp when jp is given): H(:,j) = h1 +
+// h2, H(j+1,j) = sqrt(nrm2), Givens rotations, residual estimate st->rel =
+// |g_{j+1}| / bnorm, written to host_rel (with the breakdown flag) when that
+// is not null; then the loop's step.  Cg...: the CG recurrence's scalars.
+struct Tail {
+  enum What { None, Arnoldi, CgStart, CgAlpha, CgRel, CgFirst, CgBeta };
+  What what = None;
+  ArnoldiState* st = nullptr;
+  CgState* cg = nullptr;
+  int j = 0;
+  const int* jp = nullptr;
+  double* host_rel = nullptr;
+  LoopStep loop;
 };
 Reducer make_reducer(DeviceArena& a);
 
@@ -258,14 +296,16 @@ void cheb_zero(const T* b, const T* d, T* r, T* dv, T* x, double inv_theta, long
 // out = ||x||^2 (device scalar).  Vector kernels take T = double or float;
 // FP32 vectors are summed per thread in FP32, across threads in FP64.
 template <typename T>
-void norm2(const T* x, long long n, double* out, const Reducer& r, cudaStream_t s);
+void norm2(const T* x, long long n, double* out, const Reducer& r, cudaStream_t s, const Tail& t = Tail());
 // The Gram-Schmidt and update kernels take their count k from the host, or,
 // with kp given (loops recorded in a CUDA graph), from the device as
 // *kp + koff, with k then an upper bound of it.
-// out[j] = V_j . w, j < k (V vectors of length n with stride ld)
+// out[j] = V_j . w, j < k (V vectors of length n with stride ld); with keep,
+// also column k - 1 of kept = keep
 template <typename T>
 void multidot(const T* V, long long ld, int k, const T* w, long long n, double* out, const Reducer& r,
-              cudaStream_t s, const int* kp = nullptr, int koff = 0);
+              cudaStream_t s, const int* kp = nullptr, int koff = 0, const Tail& t = Tail(), const T* keep = nullptr,
+              T* kept = nullptr);
 // w -= sum_j V_j h[j]; then out[j] = V_j . w (second Gram-Schmidt pass)
 template <typename T>
 void cgs_update_dot(const T* V, long long ld, int k, const double* h, T* w, long long n, double* out,
@@ -273,23 +313,18 @@ void cgs_update_dot(const T* V, long long ld, int k, const double* h, T* w, long
 // w -= sum_j V_j h[j]; then out = ||w||^2
 template <typename T>
 void cgs_update_norm(const T* V, long long ld, int k, const double* h, T* w, long long n, double* out,
-                     const Reducer& r, cudaStream_t s, const int* kp = nullptr, int koff = 0);
-// Arnoldi bookkeeping for column j (or *jp when jp is given): H(:,j) = h1 + h2,
-// H(j+1,j) = sqrt(nrm2), Givens rotations, residual estimate
-// st->rel = |g_{j+1}| / bnorm, copied to *host_rel (mapped host memory) when
-// host_rel is not null.
-void arnoldi_finalize(ArnoldiState* st, int j, double* host_rel, cudaStream_t s, const int* jp = nullptr);
+                     const Reducer& r, cudaStream_t s, const int* kp = nullptr, int koff = 0,
+                     const Tail& t = Tail());
 // GMRES start: beta = sqrt(st->nrm2); g = beta e_1; bnorm set when first;
 // writes beta/bnorm to *host_rel when it is not null
 void arnoldi_start(ArnoldiState* st, int first, double* host_rel, cudaStream_t s);
 // y = x * (*scale) with scale a device scalar
 template <typename T>
 void scale_by(const T* x, const double* scale, T* y, long long n, cudaStream_t s);
-// y = x (times *sc when sc is not null); x is column *xj of X when xj is
-// given, y column *yj + yoff of Y when yj is given (columns ld apart)
+// y = column *yj + yoff of Y (Y itself without yj) = (*sc) x, and z = y
 template <typename T>
-void col_copy(const T* X, const int* xj, T* Y, const int* yj, int yoff, long long ld, const double* sc, long long n,
-              cudaStream_t s);
+void scale_two(const T* x, const double* sc, T* Y, const int* yj, int yoff, long long ld, T* z, long long n,
+               cudaStream_t s);
 // y = H^{-1} g (k x k upper triangle, k = *kp when kp is given), then
 // x += sum_j y_j Z_j
 template <typename T>
@@ -297,9 +332,6 @@ void gmres_update(ArnoldiState* st, int k, const T* Z, long long ld, T* x, long 
                   const int* kp = nullptr);
 
 // CG helpers: scalars on the device
-struct CgState {
-  double rz, rz_new, pq, alpha, beta, rr, bnorm2, rel;
-};
 void cg_step_x_r(CgState* st, const double* p, const double* q, double* x, double* r, long long n,
                  const Reducer& red, double* host_rel, cudaStream_t s);
 void cg_dot_rz(CgState* st, const double* r, const double* z, long long n, const Reducer& red,

@@ -749,6 +749,31 @@ struct Hierarchy {
     gsize = sizeof(T);
   }
 
+  // true when V-cycles are replayed from the recorded graph (recorded here at
+  // first): input() and output() are then its vectors, replay() one V-cycle
+  // from the first to the second.  The per-launch event profiler needs the
+  // launches themselves.
+  template <typename T>
+  bool replays(cudaStream_t s) {
+    if (g_capture_depth > 0 || !use_graph || graph_failed || profiler().active) return false;
+    if (!gexec) capture<T>(s);
+    return gexec && gsize == sizeof(T);
+  }
+  template <typename T>
+  T* input() const {
+    return static_cast<T*>(gin);
+  }
+  template <typename T>
+  T* output() const {
+    return static_cast<T*>(gout);
+  }
+  void replay(cudaStream_t s) {
+    ++vcycles;
+    SCR_CUDA(cudaGraphLaunch(gexec.get(), s));
+    counters().launches += glaunches;
+    counters().spmv_bytes += gbytes;
+  }
+
   template <typename T>
   void apply(const T* b, T* x, cudaStream_t s) {
     if (g_capture_depth > 0) {  // recorded into a graph: counted at each replay
@@ -756,20 +781,14 @@ struct Hierarchy {
       counters().vcycles[slot]++;
       return;
     }
-    ++vcycles;
-    // the per-launch event profiler needs the launches themselves
-    if (use_graph && !graph_failed && !profiler().active) {
-      if (!gexec) capture<T>(s);
-      if (gexec && gsize == sizeof(T)) {
-        const long long n = lv[0].n * nrhs;
-        copy<T>(b, static_cast<T*>(gin), n, s);
-        SCR_CUDA(cudaGraphLaunch(gexec.get(), s));
-        copy<T>(static_cast<const T*>(gout), x, n, s);
-        counters().launches += glaunches;
-        counters().spmv_bytes += gbytes;
-        return;
-      }
+    if (replays<T>(s)) {
+      const long long n = lv[0].n * nrhs;
+      copy<T>(b, input<T>(), n, s);
+      replay(s);
+      copy<T>(output<T>(), x, n, s);
+      return;
     }
+    ++vcycles;
     cycle<T>(0, b, x, s);
   }
 };
@@ -785,16 +804,6 @@ struct Hierarchy {
 // both run the same kernels on the same data.  Every Arnoldi step counts
 // against the iteration cap and every cycle against a cycle cap, so each
 // loop ends after at most maxit body runs whatever the estimates are.
-struct KrylovLoop {
-  int j;          // Arnoldi step inside the current cycle
-  int iters;      // Arnoldi steps of the current solve
-  int cycles;     // restart cycles of the current solve
-  int nonfinite;  // 1 when an estimate was NaN or infinite
-  double rel;     // last residual estimate
-  // since the last reset (read back once per outer solve for the counters)
-  long long tot_iters, tot_solves, tot_cycles, tot_restarts;
-};
-
 // streams that record conditional bodies, one per nesting depth, created
 // before the outermost capture begins
 constexpr int kMaxCaptureDepth = 8;
@@ -815,22 +824,6 @@ __global__ void k_loop_arm(KrylovLoop* L, cudaGraphConditionalHandle h_inner) {
   L->j = 0;
   L->tot_cycles++;
   cudaGraphSetConditional(h_inner, 1u);
-}
-__global__ void k_loop_next(const ArnoldiState* __restrict__ st, KrylovLoop* L, cudaGraphConditionalHandle h_inner,
-                            double tol, int m, int maxit) {
-  const int j = L->j + 1, it = L->iters + 1;
-  L->j = j;
-  L->iters = it;
-  L->tot_iters++;
-  const double r = st->rel;
-  L->rel = r;
-  const bool fin = isfinite(r);
-  if (!fin) {  // the host loop returns here without the update: a zero count skips it
-    L->nonfinite = 1;
-    L->j = 0;
-  }
-  const bool go = fin && !(r <= tol) && st->breakdown == 0 && j < m && it < maxit;
-  cudaGraphSetConditional(h_inner, go ? 1u : 0u);
 }
 __global__ void k_loop_after(const ArnoldiState* __restrict__ st, KrylovLoop* L, cudaGraphConditionalHandle h_outer,
                              cudaGraphConditionalHandle h_restart, double tol, int maxit) {
@@ -984,7 +977,7 @@ struct Gmres {
     fill<T>(x, (T)0, n, cs);
     norm2<T>(b, n, &st->nrm2, red, cs);
     arnoldi_start(st, 1, nullptr, cs);
-    scale_by<T>(b, &st->inv_hnext, V, n, cs);
+    scale_two<T>(b, &st->inv_hnext, V, nullptr, 0, n, pin, n, cs);
     const cudaGraphConditionalHandle h_outer = make_handle(capturing_graph(cs));
     k_loop_begin<<<1, 1, 0, cs>>>(st, L, h_outer);
     SCR_LAUNCH();
@@ -1000,18 +993,20 @@ struct Gmres {
       const LaunchCounter arm = diff(counters(), c1);
       record_conditional(os, h_inner, cudaGraphCondTypeWhile, [&](cudaStream_t is) {
         const LaunchCounter c2 = counters();
-        col_copy<T>(V, &L->j, pin, nullptr, 0, n, nullptr, n, is);
+        // pin holds v_j: written with it at the end of the step before
         pc(pin, pout, is);
-        col_copy<T>(pout, nullptr, Z, &L->j, 0, n, nullptr, n, is);
         op(pout, w, is);
-        multidot<T>(V, n, m, w, n, st->h1, red, is, &L->j, 1);
+        multidot<T>(V, n, m, w, n, st->h1, red, is, &L->j, 1, Tail(), pout, Z);  // and z_j = pout
         cgs_update_dot<T>(V, n, m, st->h1, w, n, st->h2, red, is, &L->j, 1);
-        cgs_update_norm<T>(V, n, m, st->h2, w, n, &st->nrm2, red, is, &L->j, 1);
-        arnoldi_finalize(st, 0, nullptr, is, &L->j);
-        col_copy<T>(w, nullptr, V, &L->j, 1, n, &st->inv_hnext, n, is);
-        k_loop_next<<<1, 1, 0, is>>>(st, L, h_inner, tol, m, maxit);
-        SCR_LAUNCH();
-        counters().launches++;
+        Tail t;
+        t.what = Tail::Arnoldi;
+        t.st = st;
+        t.jp = &L->j;
+        t.loop = LoopStep{L, h_inner, tol, m, maxit};
+        cgs_update_norm<T>(V, n, m, st->h2, w, n, &st->nrm2, red, is, &L->j, 1, t);
+        // L->j counts the step by now (0 after a non-finite estimate, whose
+        // column nobody reads)
+        scale_two<T>(w, &st->inv_hnext, V, &L->j, 0, n, pin, n, is);
         sec[1] = diff(counters(), c2);
       });
       const LaunchCounter c3 = counters();
@@ -1027,7 +1022,7 @@ struct Gmres {
         axpby_t<T>(1.0, b, -1.0, w, n, rs);
         norm2<T>(w, n, &st->nrm2, red, rs);
         arnoldi_start(st, 0, nullptr, rs);
-        scale_by<T>(w, &st->inv_hnext, V, n, rs);
+        scale_two<T>(w, &st->inv_hnext, V, nullptr, 0, n, pin, n, rs);
         sec[3] = diff(counters(), c4);
       });
     });
@@ -1059,9 +1054,25 @@ struct Gmres {
 
   using Op = std::function<void(const T*, T*)>;
 
-  // returns true when converged; iters/rel report the work done
+  // returns true when converged; iters/rel report the work done.  hier: the
+  // hierarchy whose V-cycle pc is, if it is one: replayed from its graph, the
+  // V-cycle takes v_j where the step before left it and its result is stored
+  // as z_j by the first Gram-Schmidt pass, without copies of their own (op
+  // must not use that hierarchy)
   bool solve(const Op& op, const Op* pc, const T* b, T* x, double tol, int maxit, const Reducer& red,
-             cudaStream_t s, int* iters, double* rel, const std::function<double(const T*)>* true_rel = nullptr) {
+             cudaStream_t s, int* iters, double* rel, const std::function<double(const T*)>* true_rel = nullptr,
+             Hierarchy* hier = nullptr) {
+    T* in = nullptr;
+    T* out = nullptr;
+    if (hier && hier->template replays<T>(s)) {
+      in = hier->template input<T>();
+      out = hier->template output<T>();
+    }
+    auto basis = [&](const T* from, int j) {  // v_j = from / its norm
+      T* v = V + (size_t)j * n;
+      if (in) scale_two<T>(from, &st->inv_hnext, v, nullptr, 0, n, in, n, s);
+      else scale_by<T>(from, &st->inv_hnext, v, n, s);
+    };
     fill<T>(x, (T)0, n, s);
     norm2<T>(b, n, &st->nrm2, red, s);
     arnoldi_start(st, 1, hs.d, s);
@@ -1075,7 +1086,7 @@ struct Gmres {
       return false;
     }
     if (!(hs.h[1] > 0.0)) return true;  // b = 0 -> x = 0
-    scale_by<T>(b, &st->inv_hnext, V, n, s);
+    basis(b, 0);
     for (;;) {
       int k = 0;
       bool breakdown = false;
@@ -1083,14 +1094,24 @@ struct Gmres {
       for (int j = 0; j < m; ++j) {
         T* vj = V + (size_t)j * n;
         T* zj = Z + (size_t)j * n;
-        if (pc) (*pc)(vj, zj);
-        else copy<T>(vj, zj, n, s);
-        op(zj, w);
-        multidot<T>(V, n, j + 1, w, n, st->h1, red, s);
+        if (in) {
+          hier->replay(s);
+          op(out, w);
+          multidot<T>(V, n, j + 1, w, n, st->h1, red, s, nullptr, 0, Tail(), out, Z);
+        } else {
+          if (pc) (*pc)(vj, zj);
+          else copy<T>(vj, zj, n, s);
+          op(zj, w);
+          multidot<T>(V, n, j + 1, w, n, st->h1, red, s);
+        }
         cgs_update_dot<T>(V, n, j + 1, st->h1, w, n, st->h2, red, s);
-        cgs_update_norm<T>(V, n, j + 1, st->h2, w, n, &st->nrm2, red, s);
-        arnoldi_finalize(st, j, hs.d, s);
-        scale_by<T>(w, &st->inv_hnext, V + (size_t)(j + 1) * n, n, s);
+        Tail t;
+        t.what = Tail::Arnoldi;
+        t.st = st;
+        t.j = j;
+        t.host_rel = hs.d;
+        cgs_update_norm<T>(V, n, j + 1, st->h2, w, n, &st->nrm2, red, s, nullptr, 0, t);
+        basis(w, j + 1);
         hs.fetch(s);
         SCR_CUDA(cudaStreamSynchronize(s));
         ++syncs;
@@ -1120,7 +1141,7 @@ struct Gmres {
       axpby_t<T>(1.0, b, -1.0, w, n, s);
       norm2<T>(w, n, &st->nrm2, red, s);
       arnoldi_start(st, 0, hs.d, s);
-      scale_by<T>(w, &st->inv_hnext, V, n, s);
+      basis(w, 0);
     }
   }
 };
@@ -1365,7 +1386,7 @@ struct StreamSwap {
 // else the host-driven loop (returns its steps)
 template <typename T>
 int gmres_run(scr_ctx* h, Gmres<T>* g, const typename Gmres<T>::OpS& op, const typename Gmres<T>::OpS& pc,
-              const T* b, T* x, double tol, int maxit) {
+              const T* b, T* x, double tol, int maxit, Hierarchy* hier) {
   if (g_capture_depth > 0) {
     g->emit(h->s, op, pc, b, x, tol, maxit, h->red);
     return 0;
@@ -1375,7 +1396,7 @@ int gmres_run(scr_ctx* h, Gmres<T>* g, const typename Gmres<T>::OpS& op, const t
   typename Gmres<T>::Op p = [&](const T* a, T* y) { pc(a, y, s); };
   int it = 0;
   double rel = 0;
-  g->solve(o, &p, b, x, tol, maxit, h->red, s, &it, &rel);
+  g->solve(o, &p, b, x, tol, maxit, h->red, s, &it, &rel, nullptr, hier);
   return it;
 }
 
@@ -1446,7 +1467,7 @@ int solve_A(scr_ctx* h, PcView<T>& v, Gmres<T>* g, int k, double rtol, int maxit
     apply_A<T>(h, v, xx, y);
   };
   typename Gmres<T>::OpS pcA = [&](const T* bb, T* xx, cudaStream_t cs) { v.hA->template apply<T>(bb, xx, cs); };
-  return gmres_run<T>(h, g, opA, pcA, b, x, rtol, maxit);
+  return gmres_run<T>(h, g, opA, pcA, b, x, rtol, maxit, v.hA);
 }
 
 // Algorithm 2: y_p = D x_p - C A^{-1} (B x_p), A^{-1} by inner GMRES + P_I
@@ -1485,7 +1506,7 @@ void apply_pc(scr_ctx* h, PcView<T>& v, const T* r, T* y) {
   e.z = rp;
   spmv<T, T>(*v.C, v.yhat, v.rp2, h->k, e, s);
   // 3. S y_p = r_p
-  h->stats.s_iters += gmres_run<T>(h, v.gS, opS, pcS, v.rp2, yp, h->o.rtol_S, h->o.max_S);
+  h->stats.s_iters += gmres_run<T>(h, v.gS, opS, pcS, v.rp2, yp, h->o.rtol_S, h->o.max_S, v.hS);
   // 4. r_v <- r_v - B y_p
   e.z = rv;
   spmv<T, T>(*v.B, yp, v.rv2, h->k, e, s);
@@ -1518,7 +1539,7 @@ void apply_simple(scr_ctx* h, PcView<T>& v, const T* r, T* y) {
   e.beta = 1.0;
   e.z = rp;
   spmv<T, T>(*v.C, v.yhat, v.rp2, h->k, e, s);
-  h->stats.s_iters += gmres_run<T>(h, v.gS, opS, pcS, v.rp2, yp, h->o.rtol_S, h->o.max_S);
+  h->stats.s_iters += gmres_run<T>(h, v.gS, opS, pcS, v.rp2, yp, h->o.rtol_S, h->o.max_S, v.hS);
   EpiArgs u;
   u.kind = Epi::ScaledSub;
   u.z = v.yhat;
