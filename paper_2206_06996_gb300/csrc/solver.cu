@@ -1953,8 +1953,8 @@ int scr_setup(scr_handle h, const scr_bsr* A, const scr_bsr* B, const scr_bsr* C
     lr.set(lS, h->Shat);
     lr.set(lB, h->B);
     lr.set(lC, h->C);
-    tune_product<double>(h->A, 1, h->o, a, s);
-    tune_product<double>(h->Shat, 1, h->o, a, s);
+    tune_product<double>(h->A, h->k, h->o, a, s);
+    tune_product<double>(h->Shat, h->k, h->o, a, s);
     if (f32) {
       h->Af = float_copy(h->A, a, s);
       if (h->o.vec) build_vec<float>(h->Af, a, s);
@@ -1968,7 +1968,7 @@ int scr_setup(scr_handle h, const scr_bsr* A, const scr_bsr* B, const scr_bsr* C
         build_sell<float>(h->A, h->Af_sell, a, s, h->o.sell);
         h->Af.sell = &h->Af_sell;
       }
-      tune_product<float>(h->Af, 1, h->o, a, s);
+      tune_product<float>(h->Af, h->k, h->o, a, s);
     }
     if (h->o.verbose)
       fprintf(stderr, "[setup] lane groups: A %d, Shat %d, A(fp32) %d\n", h->A.g, h->Shat.g, h->Af.g);

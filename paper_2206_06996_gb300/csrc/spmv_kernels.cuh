@@ -1,7 +1,6 @@
-// Product kernels with G lanes per scalar row and their launch dispatch,
-// shared by the translation units that instantiate them: spmv.cu (one and
-// three right-hand sides) and spmm.cu (eight right-hand sides, the block
-// product of the multi-right-hand-side solve).
+// Product kernels of one and three right-hand sides and their launch dispatch
+// (spmv.cu), with the parts that the products of eight right-hand sides share
+// (spmm.cu).
 #pragma once
 #include <cuda_bf16.h>
 
@@ -434,6 +433,15 @@ __device__ __forceinline__ void ldg16(const VT* p, VT* a) {
     const double2 v = __ldg(reinterpret_cast<const double2*>(p));
     a[0] = v.x, a[1] = v.y;
   }
+}
+// 16 bytes of a vector (ordinary loads)
+__device__ __forceinline__ void load16(const float* p, float* a) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  a[0] = v.x, a[1] = v.y, a[2] = v.z, a[3] = v.w;
+}
+__device__ __forceinline__ void load16(const double* p, double* a) {
+  const double2 v = *reinterpret_cast<const double2*>(p);
+  a[0] = v.x, a[1] = v.y;
 }
 template <int U>
 __device__ __forceinline__ void ldg_idx(const int* p, int* c) {
