@@ -250,18 +250,24 @@ void l1_inv(const DBsr<double>& A, double* dinv, cudaStream_t s) {
   counters().launches++;
 }
 
+// A thread sums its row in order: another order would move the bound by an
+// ulp, and with it the values that the truncation of the prolongators compares
+// (rows of symmetric meshes hold exact ties).
 __global__ void k_gershgorin(DBsr<double> A, const double* __restrict__ d, unsigned long long* __restrict__ out) {
   const long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long n = (long long)A.nbr * A.br;
-  if (o >= n) return;
-  const int i = (int)(o / A.br), r = (int)(o - (long long)i * A.br);
-  const int s = A.rp[i], k = A.rp[i + 1] - s, L = k * A.bc;
-  const double* v = A.val + (long long)s * A.br * A.bc + (long long)r * L;
-  double acc = 0.0;
-  for (int q = 0; q < L; ++q) acc += fabs(v[q]);
-  const double ratio = acc / fabs(d[o]);
-  // non-negative doubles order like their bit patterns
-  atomicMax(out, (unsigned long long)__double_as_longlong(ratio));
+  unsigned long long b = 0;
+  if (o < n) {
+    const int i = (int)(o / A.br), r = (int)(o - (long long)i * A.br);
+    const int s = A.rp[i], k = A.rp[i + 1] - s, L = k * A.bc;
+    const double* v = A.val + (long long)s * A.br * A.bc + (long long)r * L;
+    double acc = 0.0;
+    for (int q = 0; q < L; ++q) acc += fabs(v[q]);
+    // non-negative doubles order like their bit patterns
+    b = (unsigned long long)__double_as_longlong(acc / fabs(d[o]));
+  }
+  for (int w = 16; w > 0; w >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, w));
+  if ((threadIdx.x & 31) == 0) atomicMax(out, b);
 }
 
 void gershgorin(const DBsr<double>& A, const double* d, double* out, cudaStream_t s) {
@@ -311,46 +317,63 @@ void scale_rows_inv(const DBsr<double>& M, const double* d, DBsr<double>& out, D
 }
 
 // ------------------------------------------------------------ strength
+// Passes over a row's entries take kRowLanes lanes per row: one thread per row
+// walked 15 to 80 entries with a dependent search each.
+constexpr int kRowLanes = 8;
+
 __global__ void k_block_norms(DBsr<double> A, double* __restrict__ bnorm, double* __restrict__ dnorm) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= A.nbr) return;
-  const int s = A.rp[i], k = A.rp[i + 1] - s;
+  const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const int i = (int)(g / kRowLanes), lane = (int)(g % kRowLanes);
   double dn = 0.0;
-  for (int t = 0; t < k; ++t) {
-    double acc = 0.0;
-    for (int r = 0; r < A.br; ++r)
-      for (int c = 0; c < A.bc; ++c) {
-        const double v = A.val[slab_index(s, k, t, r, c, A.br, A.bc)];
-        acc += v * v;
+  bool found = false;
+  if (i < A.nbr) {
+    const int s = A.rp[i], k = A.rp[i + 1] - s;
+    for (int t = lane; t < k; t += kRowLanes) {
+      double acc = 0.0;
+      for (int r = 0; r < A.br; ++r)
+        for (int c = 0; c < A.bc; ++c) {
+          const double v = A.val[slab_index(s, k, t, r, c, A.br, A.bc)];
+          acc += v * v;
+        }
+      const double nv = sqrt(acc);
+      bnorm[s + t] = nv;
+      if (A.col[s + t] == i) {
+        dn = nv;
+        found = true;
       }
-    const double nv = sqrt(acc);
-    bnorm[s + t] = nv;
-    if (A.col[s + t] == i) dn = nv;
+    }
   }
-  dnorm[i] = dn;
+  const unsigned m = __ballot_sync(0xffffffffu, found);
+  const int l0 = (threadIdx.x & 31) / kRowLanes * kRowLanes;
+  const bool any = (m >> l0) & ((1u << kRowLanes) - 1);
+  if (i < A.nbr && (any ? found : lane == 0)) dnorm[i] = dn;
 }
 
 __global__ void k_strong(DBsr<double> A, const double* __restrict__ bnorm, const double* __restrict__ dnorm,
                          double theta, unsigned char* __restrict__ strong, int* __restrict__ cnt) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= A.nbr) return;
-  const int s = A.rp[i], e = A.rp[i + 1];
+  const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const int i = (int)(g / kRowLanes), lane = (int)(g % kRowLanes);
   int c = 0;
-  for (int t = s; t < e; ++t) {
-    const int j = A.col[t];
-    unsigned char f = 0;
-    if (j != i) {
-      const double thr = theta * sqrt(dnorm[i] * dnorm[j]);
-      if (bnorm[t] > 0.0 && bnorm[t] >= thr) f = 1;
-      // transpose entry (j, i)
-      const int sj = A.rp[j], ej = A.rp[j + 1];
-      const int p = find_in_row(A.col, sj, ej, i);
-      if (p < ej && A.col[p] == i && bnorm[p] > 0.0 && bnorm[p] >= thr) f = 1;
+  if (i < A.nbr) {
+    const int s = A.rp[i], e = A.rp[i + 1];
+    for (int t = s + lane; t < e; t += kRowLanes) {
+      const int j = A.col[t];
+      unsigned char f = 0;
+      if (j != i) {
+        const double thr = theta * sqrt(dnorm[i] * dnorm[j]);
+        if (bnorm[t] > 0.0 && bnorm[t] >= thr) f = 1;
+        if (!f) {  // transpose entry (j, i)
+          const int sj = A.rp[j], ej = A.rp[j + 1];
+          const int p = find_in_row(A.col, sj, ej, i);
+          if (p < ej && A.col[p] == i && bnorm[p] > 0.0 && bnorm[p] >= thr) f = 1;
+        }
+      }
+      strong[t] = f;
+      c += f;
     }
-    strong[t] = f;
-    c += f;
   }
-  cnt[i] = c;
+  c = warp_sum(c, kRowLanes);
+  if (i < A.nbr && lane == 0) cnt[i] = c;
 }
 
 __global__ void k_strong_fill(DBsr<double> A, const unsigned char* __restrict__ strong,
@@ -489,9 +512,10 @@ Aggregation aggregate(const DBsr<double>& A, double theta, DeviceArena& arena, D
   unsigned char* strong = tmp.alloc<unsigned char>(A.nnzb);
   int* cnt = tmp.alloc<int>(n + 1);
   int* srp = tmp.alloc<int>(n + 1);
-  k_block_norms<<<G, T, 0, s>>>(A, bnorm, dnorm);
+  const int GR = ceil_div((long long)n * kRowLanes, T);
+  k_block_norms<<<GR, T, 0, s>>>(A, bnorm, dnorm);
   SCR_LAUNCH();
-  k_strong<<<G, T, 0, s>>>(A, bnorm, dnorm, theta, strong, cnt);
+  k_strong<<<GR, T, 0, s>>>(A, bnorm, dnorm, theta, strong, cnt);
   SCR_LAUNCH();
   const long long ns = exclusive_scan(cnt, srp, n, tmp, s);
   int* snb = tmp.alloc<int>(ns + 1);
@@ -611,12 +635,15 @@ __global__ void k_spgemm_ub(DBsr<double> A, DBsr<double> B, int* __restrict__ ub
   ub[i] = (int)min(u, (long long)0x3fffffff);
 }
 
-// table size for a row with upper bound ub (0: shared-memory table)
-__device__ __forceinline__ int global_table_size(int ub) {
-  if (ub <= kHashSlots / 2) return 0;
-  int g = 1;
-  while (g < 2 * ub && g < kGlobalSlots) g <<= 1;
-  return g;
+// rows whose table fits the warp's shared memory
+__device__ __forceinline__ bool small_row(int ub) { return ub <= kHashSlots / 2; }
+// slots for a row of at most ub distinct columns: twice as many, at least a
+// warp's width.  (A table of kHashSlots for every row made clearing and
+// scanning it the symbolic passes' main work: rows of 5 to 80 entries, 556 us
+// per fill on average on the bench tube's products.)
+__device__ __forceinline__ int table_size(int ub) {
+  const int want = min(2 * max(ub, 1), kGlobalSlots);
+  return max(32, 1 << (32 - __clz(want - 1)));
 }
 
 // insert the columns of row i of A*B into a warp's hash table; returns the
@@ -665,37 +692,52 @@ __device__ int spgemm_insert(const DBsr<double>& A, const DBsr<double>& B, int i
   return mine;
 }
 
-__global__ void __launch_bounds__(32 * kSpgemmWarps) k_spgemm_count(DBsr<double> A, DBsr<double> B,
-                                                                   const int* __restrict__ ub, int* __restrict__ gtab,
-                                                                   int* __restrict__ cnt, int* __restrict__ err) {
+// Rows of a symbolic pass: the first `big` CTAs take the rows whose tables do
+// not fit shared memory (each warp looks through every big * kSpgemmWarps-th
+// group of 32 rows), the others one small row per warp.  body(i, table, size)
+// runs with all lanes of a warp.
+template <class F>
+__device__ __forceinline__ void spgemm_rows(int n, const int* __restrict__ ub, int big, int* gtab, F&& body) {
   __shared__ int smem[kSpgemmWarps][kHashSlots];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int gw = blockIdx.x * kSpgemmWarps + w, nw = gridDim.x * kSpgemmWarps;
-  int* gtab_w = gtab + (long long)gw * kGlobalSlots;
-  for (int i = gw; i < A.nbr; i += nw) {
-    const int gs = global_table_size(ub[i]);
-    int* table = gs ? gtab_w : smem[w];
-    const int hsize = gs ? gs : kHashSlots;
+  if ((int)blockIdx.x >= big) {
+    const int i = (blockIdx.x - big) * kSpgemmWarps + w;
+    if (i < n && small_row(ub[i])) body(i, smem[w], table_size(ub[i]));
+    return;
+  }
+  const int gw = blockIdx.x * kSpgemmWarps + w, nw = big * kSpgemmWarps;
+  int* table = gtab + (long long)gw * kGlobalSlots;
+  for (long long r0 = 32LL * gw; r0 < n; r0 += 32LL * nw) {
+    unsigned m = __ballot_sync(0xffffffffu, r0 + lane < n && !small_row(ub[r0 + lane]));
+    while (m) {
+      const int i = (int)r0 + __ffs(m) - 1;
+      m &= m - 1;
+      body(i, table, table_size(ub[i]));
+    }
+  }
+}
+
+__global__ void __launch_bounds__(32 * kSpgemmWarps) k_spgemm_count(DBsr<double> A, DBsr<double> B,
+                                                                   const int* __restrict__ ub, int big,
+                                                                   int* __restrict__ gtab, int* __restrict__ cnt,
+                                                                   int* __restrict__ err) {
+  spgemm_rows(A.nbr, ub, big, gtab, [&](int i, int* table, int hsize) {
+    const int lane = threadIdx.x & 31;
     for (int h = lane; h < hsize; h += 32) table[h] = -1;
     __syncwarp();
     const int mine = spgemm_insert(A, B, i, ub[i], table, hsize, lane, err);
     const int tot = warp_sum(mine);
     if (lane == 0) cnt[i] = tot;
     __syncwarp();
-  }
+  });
 }
 
 __global__ void __launch_bounds__(32 * kSpgemmWarps) k_spgemm_fill(DBsr<double> A, DBsr<double> B,
-                                                                  const int* __restrict__ ub, int* __restrict__ gtab,
-                                                                  DBsr<double> C, int* __restrict__ err) {
-  __shared__ int smem[kSpgemmWarps][kHashSlots];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int gw = blockIdx.x * kSpgemmWarps + w, nw = gridDim.x * kSpgemmWarps;
-  int* gtab_w = gtab + (long long)gw * kGlobalSlots;
-  for (int i = gw; i < A.nbr; i += nw) {
-    const int gs = global_table_size(ub[i]);
-    int* table = gs ? gtab_w : smem[w];
-    const int hsize = gs ? gs : kHashSlots;
+                                                                  const int* __restrict__ ub, int big,
+                                                                  int* __restrict__ gtab, DBsr<double> C,
+                                                                  int* __restrict__ err) {
+  spgemm_rows(A.nbr, ub, big, gtab, [&](int i, int* table, int hsize) {
+    const int lane = threadIdx.x & 31;
     for (int h = lane; h < hsize; h += 32) table[h] = -1;
     __syncwarp();
     spgemm_insert(A, B, i, ub[i], table, hsize, lane, err);
@@ -722,29 +764,36 @@ __global__ void __launch_bounds__(32 * kSpgemmWarps) k_spgemm_fill(DBsr<double> 
       C.col[base + rank] = v;
     }
     __syncwarp();
-  }
+  });
 }
 
+// Values of C = A B on C's pattern, a warp per row.
 template <int BR, int BK, int BC>
 __global__ void __launch_bounds__(32 * kSpgemmWarps) k_spgemm_numeric(DBsr<double> A, DBsr<double> B,
                                                                      DBsr<double> C) {
+  constexpr int NE = BR * BC;
+  constexpr int kCap = NE == 9 ? 64 : kNumericCols;  // output entries of the product-parallel path
+  __shared__ int ccol[kSpgemmWarps][kCap];
+  __shared__ double sums[kSpgemmWarps][kCap * NE], prods[kSpgemmWarps][32 * NE];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * kSpgemmWarps + w;
   if (i >= A.nbr) return;  // uniform over the warp
   const int cs = C.rp[i], ck = C.rp[i + 1] - cs;
-  double* cv = C.val + (long long)cs * BR * BC;
+  double* cv = C.val + (long long)cs * NE;
   const int as = A.rp[i], ak = A.rp[i + 1] - as;
-  if (ck <= 32) {
-    // Rows with at most 32 output entries (the prolongator and Galerkin
-    // products): A's row is taken in chunks of 32 entries; within a chunk
-    // the partial products (t, u) = (entry t of A's row, entry u of the B row
-    // it selects) are numbered p in t-major order, lane p % 32 forms product
-    // p, and lane e, owner of output entry e, adds the products that land on
-    // e in increasing t, i.e. in the order of the general path below.
-    constexpr unsigned kFull = 0xffffffffu;
-    double acc[BR * BC];
-#pragma unroll
-    for (int e = 0; e < BR * BC; ++e) acc[e] = 0.0;
+  constexpr unsigned kFull = 0xffffffffu;
+  if (ck <= kCap) {
+    // A's row is taken in chunks of 32 entries; within a chunk the partial
+    // products (t, u) = (entry t of A's row, entry u of the B row it selects)
+    // are numbered p in t-major order and formed 32 at a time, one per lane.
+    // Of the products that land on one output entry the first one's lane adds
+    // them in increasing p, which is the order of the general path below, so
+    // the lanes add to as many outputs at once as the 32 products have.
+    // (Adding product by product, with one lane of the FP64 pipe in use, took
+    // 1.3 ms on average for the bench tube's 3x3 products.)
+    for (int e = lane; e < ck; e += 32) ccol[w][e] = C.col[cs + e];
+    for (int e = lane; e < ck * NE; e += 32) sums[w][e] = 0.0;
+    __syncwarp();
     for (int tc = 0; tc < ak; tc += 32) {
       const int nt = min(32, ak - tc);
       int bst = 0, lent = 0;
@@ -759,22 +808,25 @@ __global__ void __launch_bounds__(32 * kSpgemmWarps) k_spgemm_numeric(DBsr<doubl
         const int v = __shfl_up_sync(kFull, incl, o);
         if (lane >= o) incl += v;
       }
-      const int off = incl - lent;
+      const int off = incl - lent;  // products before this lane's entry
       const int np = __shfl_sync(kFull, incl, 31);
       for (int base = 0; base < np; base += 32) {
         const int p = base + lane;
-        int tl = 0;  // the last entry of the chunk whose products start at or before p
-        for (int q = 1; q < nt; ++q)
-          if (__shfl_sync(kFull, off, q) <= p) tl = q;
+        // the entry whose products hold p: the number of entries that end at
+        // or before it
+        int tl = 0;
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1) {
+          const int end = __shfl_sync(kFull, incl, tl + step - 1);
+          if (end <= p) tl += step;
+        }
+        tl = min(tl, 31);
         const int j_b = __shfl_sync(kFull, bst, tl), j_len = __shfl_sync(kFull, lent, tl);
         const int u = p - __shfl_sync(kFull, off, tl);
         int pos = -1;
-        double prod[BR * BC];
-#pragma unroll
-        for (int e = 0; e < BR * BC; ++e) prod[e] = 0.0;
         if (p < np) {
           const int t = tc + tl;
-          pos = find_in_row(C.col, cs, cs + ck, B.col[j_b + u]) - cs;
+          pos = find_in_row(ccol[w], 0, ck, B.col[j_b + u]);
 #pragma unroll
           for (int r = 0; r < BR; ++r)
 #pragma unroll
@@ -784,35 +836,36 @@ __global__ void __launch_bounds__(32 * kSpgemmWarps) k_spgemm_numeric(DBsr<doubl
               for (int m = 0; m < BK; ++m)
                 v = fma(A.val[slab_index(as, ak, t, r, m, BR, BK)], B.val[slab_index(j_b, j_len, u, m, q, BK, BC)],
                         v);
-              prod[r * BC + q] = v;
+              prods[w][lane * NE + r * BC + q] = v;
             }
         }
-        const int cnt = min(32, np - base);
-        for (int q = 0; q < cnt; ++q) {
-          const int pq = __shfl_sync(kFull, pos, q);
+        unsigned same = __match_any_sync(kFull, pos);
+        __syncwarp();
+        if (pos >= 0 && pos < ck && lane == __ffs(same) - 1) {
+          double acc[NE];
 #pragma unroll
-          for (int e = 0; e < BR * BC; ++e) {
-            const double v = __shfl_sync(kFull, prod[e], q);
-            if (lane == pq) acc[e] += v;
+          for (int r = 0; r < BR; ++r)
+#pragma unroll
+            for (int q = 0; q < BC; ++q) acc[r * BC + q] = sums[w][r * ck * BC + pos * BC + q];
+          while (same) {
+            const int q = __ffs(same) - 1;
+            same &= same - 1;
+#pragma unroll
+            for (int e = 0; e < NE; ++e) acc[e] += prods[w][q * NE + e];
           }
+#pragma unroll
+          for (int r = 0; r < BR; ++r)
+#pragma unroll
+            for (int q = 0; q < BC; ++q) sums[w][r * ck * BC + pos * BC + q] = acc[r * BC + q];
         }
+        __syncwarp();
       }
     }
-    if (lane < ck) {
-#pragma unroll
-      for (int r = 0; r < BR; ++r)
-#pragma unroll
-        for (int q = 0; q < BC; ++q) cv[(long long)r * ck * BC + (long long)lane * BC + q] = acc[r * BC + q];
-    }
+    for (int e = lane; e < ck * NE; e += 32) cv[e] = sums[w][e];
     return;
   }
-  // general path: the output row's columns in shared memory when they fit,
-  // for the searches below
-  __shared__ int ccol[kSpgemmWarps][kNumericCols];
-  const bool cached = ck <= kNumericCols;
-  if (cached)
-    for (int e = lane; e < ck; e += 32) ccol[w][e] = C.col[cs + e];
-  for (int e = lane; e < ck * BR * BC; e += 32) cv[e] = 0.0;
+  // general path: the lanes share each B row, sums in C's row
+  for (int e = lane; e < ck * NE; e += 32) cv[e] = 0.0;
   __syncwarp();
   for (int t = 0; t < ak; ++t) {
     double a[BR][BK];
@@ -823,8 +876,7 @@ __global__ void __launch_bounds__(32 * kSpgemmWarps) k_spgemm_numeric(DBsr<doubl
     const int j = A.col[as + t];
     const int bs = B.rp[j], bk = B.rp[j + 1] - bs;
     for (int u = lane; u < bk; u += 32) {
-      const int c = B.col[bs + u];
-      const int pos = cached ? find_in_row(ccol[w], 0, ck, c) : find_in_row(C.col, cs, cs + ck, c) - cs;
+      const int pos = find_in_row(C.col, cs, cs + ck, B.col[bs + u]) - cs;
       if (pos >= ck) continue;  // cannot happen for a consistent symbolic phase
       double b[BK][BC];
 #pragma unroll
@@ -867,10 +919,11 @@ void spgemm(const DBsr<double>& A, const DBsr<double>& B, DBsr<double>& C, Devic
   SCR_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
   k_spgemm_ub<<<ceil_div(n, 256), 256, 0, s>>>(A, B, ub);
   SCR_LAUNCH();
-  // persistent grid: 4 blocks of 4 warps per SM, each warp owning a slice
-  const int pgrid = std::min(ceil_div(n, kSpgemmWarps), 4 * sm_count());
-  int* gtab = tmp.alloc<int>((size_t)pgrid * kSpgemmWarps * kGlobalSlots);
-  k_spgemm_count<<<pgrid, 32 * kSpgemmWarps, 0, s>>>(A, B, ub, gtab, cnt, err);
+  // CTAs for the rows with large tables, each warp with one in global memory
+  const int big = std::min(ceil_div(n, 32 * kSpgemmWarps), 2 * sm_count());
+  const int pgrid = big + ceil_div(n, kSpgemmWarps);
+  int* gtab = tmp.alloc<int>((size_t)big * kSpgemmWarps * kGlobalSlots);
+  k_spgemm_count<<<pgrid, 32 * kSpgemmWarps, 0, s>>>(A, B, ub, big, gtab, cnt, err);
   SCR_LAUNCH();
   C.nnzb = exclusive_scan(cnt, C.rp, n, tmp, s);  // synchronises
   int herr = 0;
@@ -879,7 +932,7 @@ void spgemm(const DBsr<double>& A, const DBsr<double>& B, DBsr<double>& C, Devic
   if (herr) throw CudaError{cudaErrorInvalidValue, "spgemm: a product row exceeds the hash-table capacity"};
   C.col = arena.alloc<int>(C.nnzb + 1);
   C.val = arena.alloc<double>(C.nnzb * C.br * C.bc + 1);
-  k_spgemm_fill<<<pgrid, 32 * kSpgemmWarps, 0, s>>>(A, B, ub, gtab, C, err);
+  k_spgemm_fill<<<pgrid, 32 * kSpgemmWarps, 0, s>>>(A, B, ub, big, gtab, C, err);
   SCR_LAUNCH();
   const int grid = ceil_div(n, kSpgemmWarps);
   const int br = A.br, bk = A.bc, bc = B.bc;
