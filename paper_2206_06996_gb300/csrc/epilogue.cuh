@@ -36,6 +36,8 @@ struct Epilogue {
       v.p = z[gi], v.d = dinv[o];
     } else if constexpr (E == Epi::ChebStep) {
       v.p = r[gi], v.q = xin[gi], v.t = xsol[gi], v.d = dinv[o];
+    } else if constexpr (E == Epi::ChebZero) {
+      v.d = dinv[o];
     }
     return v;
   }
@@ -59,6 +61,13 @@ struct Epilogue {
       r[gi] = ri;
       dout[gi] = di;
       y[gi] = v.q + di;
+    } else if constexpr (E == Epi::ChebZero) {
+      const XT ri = (XT)acc * v.d;
+      const XT di = ri * alpha;
+      y[gi] = (XT)acc;
+      r[gi] = ri;
+      dout[gi] = di;
+      xsol[gi] = di;
     } else {
       const XT ri = v.p - (XT)acc * v.d;
       const XT di = alpha * v.q + beta * ri;

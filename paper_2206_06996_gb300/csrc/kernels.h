@@ -68,6 +68,8 @@ enum class Epi : int {
   ChebFirst = 4,  // r = (z - acc) dinv[o]; dout = alpha r; y = xs + dout   (x = xs)
   ChebStep = 5,   // r -= acc dinv[o]; dout = alpha x + beta r; xsol += dout (x = d)
   ScaledSub = 6,  // y = z - acc * dinv[o]
+  ChebZero = 7,   // y = acc; r = acc dinv[o]; dout = xsol = alpha r   (a restriction with the coarse
+                  // level's Chebyshev start from zero)
 };
 struct EpiArgs {
   Epi kind = Epi::Set;

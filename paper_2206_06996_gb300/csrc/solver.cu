@@ -182,6 +182,10 @@ struct Hierarchy {
   // CUDA graph of one V-cycle from the staging vector gin to gout (captured
   // at the first V-cycle after set-up, replayed by every later one); the
   // library counters of one captured V-cycle are added at each replay
+  // levels of at least this many scalar rows have their products timed: on the
+  // coarse levels the heuristic's lanes were up to twice as slow as the best
+  // (2,220 rows of 17 blocks, FP64: 12 us with 16 lanes, 4 us with 4)
+  static constexpr long long kTuneRows = 256;
   bool use_graph = false, graph_failed = false;
   GraphExecPtr gexec;
   void *gin = nullptr, *gout = nullptr;
@@ -290,6 +294,15 @@ struct Hierarchy {
         lr.set(ir[l], lv[l].R);
       }
     }
+    // product kernels of the FP64 levels, before the smoother data (as above)
+    if (o.autotune && !f32)
+      for (size_t l = 0; l + 1 < lv.size(); ++l) {
+        Level& L = lv[l];
+        if (L.n < kTuneRows) continue;
+        if (l > 0 || A0.g == 0) tune_product<double>(L.A, nrhs, o, ar, s);
+        tune_product<double>(L.P, nrhs, o, ar, s);
+        tune_product<double>(L.R, nrhs, o, ar, s);
+      }
     // coarsest level: dense inverse
     Level& C = lv.back();
     nc = (int)C.n;
@@ -364,26 +377,15 @@ struct Hierarchy {
       cinvf = ar.alloc<float>((size_t)nc * nc + 1);
       cast_d2f(cinv, cinvf, (long long)nc * nc, s);
     }
-    // lane-group widths of the products on the two finest levels
-    if (o.autotune) {
-      for (size_t l = 0; l < lv.size() && l < 2; ++l) {
+    // product kernels of the FP32 levels (the FP64 ones: above)
+    if (o.autotune && f32)
+      for (size_t l = 0; l + 1 < lv.size(); ++l) {
         Level& L = lv[l];
-        if (L.n < 4096) continue;
-        if (f32) {
-          if (!(l == 0 && A0f)) tune_product<float>(L.Af, nrhs, o, ar, s);
-          if (L.P.nbr) {
-            tune_product<float>(L.Pf, nrhs, o, ar, s);
-            tune_product<float>(L.Rf, nrhs, o, ar, s);
-          }
-        } else {
-          if (l > 0 || A0.g == 0) tune_product<double>(L.A, nrhs, o, ar, s);
-          if (L.P.nbr) {
-            tune_product<double>(L.P, nrhs, o, ar, s);
-            tune_product<double>(L.R, nrhs, o, ar, s);
-          }
-        }
+        if (L.n < kTuneRows) continue;
+        if (!(l == 0 && A0f)) tune_product<float>(L.Af, nrhs, o, ar, s);
+        tune_product<float>(L.Pf, nrhs, o, ar, s);
+        tune_product<float>(L.Rf, nrhs, o, ar, s);
       }
-    }
     SCR_CUDA(cudaStreamSynchronize(s));
     settle(true);
   }
@@ -574,14 +576,9 @@ struct Hierarchy {
     *inv_theta = 1.0 / theta;
   }
 
+  // the level's Chebyshev vectors and inverse diagonal in precision T
   template <typename T>
-  void cycle_cheb(int l, const T* b, T* out, cudaStream_t s) {
-    Level& L = lv[l];
-    const DBsr<T>& A = pick<T>(L.A, L.Af);
-    const DBsr<T>& P = pick<T>(L.P, L.Pf);
-    const DBsr<T>& R = pick<T>(L.R, L.Rf);
-    const T* dd;
-    T *d0, *d1;
+  static void cheb_vectors(const Level& L, const T*& dd, T*& d0, T*& d1) {
     if constexpr (sizeof(T) == 8) {
       dd = L.dd;
       d0 = L.d0;
@@ -591,13 +588,28 @@ struct Hierarchy {
       d0 = L.d0f;
       d1 = L.d1f;
     }
+  }
+  bool cheb_level(int l) const {
+    return l + 1 < n_levels() && smoother == SCR_SMOOTH_CHEB && !lv[l].cheb_off;
+  }
+
+  // started: b's restriction has already written the start from zero
+  template <typename T>
+  void cycle_cheb(int l, const T* b, T* out, cudaStream_t s, bool started) {
+    Level& L = lv[l];
+    const DBsr<T>& A = pick<T>(L.A, L.Af);
+    const DBsr<T>& P = pick<T>(L.P, L.Pf);
+    const DBsr<T>& R = pick<T>(L.R, L.Rf);
+    const T* dd;
+    T *d0, *d1;
+    cheb_vectors<T>(L, dd, d0, d1);
     double inv_theta;
     std::vector<std::pair<double, double>> st;
     cheb_coeffs(L.lam, degree, &inv_theta, st);
     T* r = vr<T>(L);
     T* cur = vt<T>(L);
     // pre-smoothing from zero
-    cheb_zero<T>(b, dd, r, d0, cur, inv_theta, L.n, nrhs, s);
+    if (!started) cheb_zero<T>(b, dd, r, d0, cur, inv_theta, L.n, nrhs, s);
     EpiArgs e;
     e.kind = Epi::ChebStep;
     e.dinv = dd;
@@ -617,9 +629,9 @@ struct Hierarchy {
     spmv<T, T>(A, cur, r, nrhs, res, s);
     Level& Lc = lv[l + 1];
     T* bc = vb<T>(Lc);
-    spmv<T, T>(R, r, bc, nrhs, EpiArgs(), s);
+    restrict_to<T>(l + 1, R, r, bc, s);
     T* xc = vx<T>(Lc);
-    cycle<T>(l + 1, bc, xc, s);
+    cycle<T>(l + 1, bc, xc, s, true);
     EpiArgs pro;
     pro.kind = Epi::Axpby;
     pro.alpha = 1.0;
@@ -646,17 +658,39 @@ struct Hierarchy {
     }
   }
 
-  // out = V-cycle(b) at level l, starting from a zero iterate
+  // bc = R r for level l; for a Chebyshev level also its start from zero, which
+  // would be a launch of its own (2.2 us per level and V-cycle)
   template <typename T>
-  void cycle(int l, const T* b, T* out, cudaStream_t s) {
+  void restrict_to(int l, const DBsr<T>& R, const T* r, T* bc, cudaStream_t s) {
+    EpiArgs e;
+    if (cheb_level(l)) {
+      Level& L = lv[l];
+      const T* dd;
+      T *d0, *d1;
+      cheb_vectors<T>(L, dd, d0, d1);
+      std::vector<std::pair<double, double>> st;
+      e.kind = Epi::ChebZero;
+      cheb_coeffs(L.lam, degree, &e.alpha, st);
+      e.dinv = dd;
+      e.r = vr<T>(L);
+      e.dout = d0;
+      e.xsol = vt<T>(L);
+    }
+    spmv<T, T>(R, r, bc, nrhs, e, s);
+  }
+
+  // out = V-cycle(b) at level l, starting from a zero iterate; restricted: b
+  // comes from restrict_to
+  template <typename T>
+  void cycle(int l, const T* b, T* out, cudaStream_t s, bool restricted = false) {
     Level& L = lv[l];
     if (l == n_levels() - 1) {
       if constexpr (sizeof(T) == 8) dense_apply(cinv, b, out, nc, nrhs, s);
       else dense_apply_f(cinvf, b, out, nc, nrhs, s);
       return;
     }
-    if (smoother == SCR_SMOOTH_CHEB && !L.cheb_off) {
-      cycle_cheb<T>(l, b, out, s);
+    if (cheb_level(l)) {
+      cycle_cheb<T>(l, b, out, s, restricted);
       return;
     }
     const DBsr<T>& A = pick<T>(L.A, L.Af);
@@ -685,9 +719,9 @@ struct Hierarchy {
     spmv<T, T>(A, cur, r, nrhs, res, s);
     Level& Lc = lv[l + 1];
     T* bc = vb<T>(Lc);
-    spmv<T, T>(R, r, bc, nrhs, EpiArgs(), s);
+    restrict_to<T>(l + 1, R, r, bc, s);
     T* xc = vx<T>(Lc);
-    cycle<T>(l + 1, bc, xc, s);
+    cycle<T>(l + 1, bc, xc, s, true);
     EpiArgs pro;
     pro.kind = Epi::Axpby;
     pro.alpha = 1.0;

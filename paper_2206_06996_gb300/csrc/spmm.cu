@@ -102,8 +102,10 @@ static void launch_spmm_e(int G, const DBsr<VT>& M, const XT* x, XT* y, const Ep
     case Epi::ScaledSub: launch_spmm<BR, BC, VT, XT, Epi::ScaledSub>(G, M, x, y, e, s); break;
     case Epi::ChebFirst:
     case Epi::ChebStep:
+    case Epi::ChebZero:
       if constexpr (BR == BC) {
         if (e.kind == Epi::ChebFirst) launch_spmm<BR, BC, VT, XT, Epi::ChebFirst>(G, M, x, y, e, s);
+        else if (e.kind == Epi::ChebZero) launch_spmm<BR, BC, VT, XT, Epi::ChebZero>(G, M, x, y, e, s);
         else launch_spmm<BR, BC, VT, XT, Epi::ChebStep>(G, M, x, y, e, s);
       } else {
         throw CudaError{cudaErrorInvalidValue, "Chebyshev epilogue on a non-square block shape"};

@@ -383,6 +383,7 @@ void spmv(const DBsr<VT>& M, const XT* x, XT* y, int nrhs, const EpiArgs& e, cud
     if (e.kind == Epi::Jacobi) b += 2.0 * nrow * nrhs * sizeof(XT) + nrow * sizeof(XT);
     if (e.kind == Epi::ScaledSub) b += nrow * nrhs * sizeof(XT) + nrow * sizeof(XT);
     if (e.kind == Epi::ChebFirst) b += 4.0 * nrow * nrhs * sizeof(XT) + nrow * sizeof(XT);
+    if (e.kind == Epi::ChebZero) b += 3.0 * nrow * nrhs * sizeof(XT) + nrow * sizeof(XT);
     if (e.kind == Epi::ChebStep) b += 5.0 * nrow * nrhs * sizeof(XT) + nrow * sizeof(XT);
     counters().spmv_bytes += (long long)b;
     prof_stop(pidx, b, 2.0 * (double)M.nnzb * M.br * M.bc * nrhs, s);

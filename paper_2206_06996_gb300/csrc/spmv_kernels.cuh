@@ -775,8 +775,10 @@ inline void launch_spmv_e(const DBsr<VT>& M, const XT* x, XT* y, const EpiArgs& 
     case Epi::ScaledSub: launch_spmv_g<BR, BC, NRHS, G, VT, XT, AT, Epi::ScaledSub>(M, x, y, e, s); break;
     case Epi::ChebFirst:
     case Epi::ChebStep:
+    case Epi::ChebZero:
       if constexpr (BR == BC) {
         if (e.kind == Epi::ChebFirst) launch_spmv_g<BR, BC, NRHS, G, VT, XT, AT, Epi::ChebFirst>(M, x, y, e, s);
+        else if (e.kind == Epi::ChebZero) launch_spmv_g<BR, BC, NRHS, G, VT, XT, AT, Epi::ChebZero>(M, x, y, e, s);
         else launch_spmv_g<BR, BC, NRHS, G, VT, XT, AT, Epi::ChebStep>(M, x, y, e, s);
       } else {
         throw CudaError{cudaErrorInvalidValue, "Chebyshev epilogue on a non-square block shape"};
@@ -816,11 +818,13 @@ inline int pick_group(const DBsr<VT>& M) {
   // with one group per row, and their rows are long, so each lane would walk
   // dozens of blocks one dependent L2 round trip at a time: widen the group
   // (up to 16 lanes, at least 4 values per lane) while the grid stays below
-  // two waves.  Measured on the coarse tube levels: about 23 us per product
-  // with 2 lanes whatever the level's size.
+  // two waves, in FP64 below 256 lanes per SM: there every further lane of a
+  // row adds a sum on the FP64 pipe (Chebyshev step, 1,200 rows of 15 blocks:
+  // 4.9, 3.5, 2.9, 4.1 us with 2, 4, 8, 16 lanes, 6,000 rows 4.9, 5.0, 6.4,
+  // 10.6 us).
   const long long nrows = (long long)M.nbr * M.br;
-  const long long wave = (long long)sm_count() * 2048;
-  while (G < 16 && per_row >= 8.0 * G && nrows * G < wave) G *= 2;
+  const long long most = (long long)sm_count() * (sizeof(VT) == 8 ? 256 : 4096);
+  while (G < 16 && per_row >= 8.0 * G && nrows * G * 2 <= most) G *= 2;
   return G;
 }
 
