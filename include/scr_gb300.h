@@ -128,12 +128,13 @@ typedef struct {
                          scr_setup fixed (modified Newton); 1 re-assemble it on the GPU at every
                          iteration's state (scr_assemble_tangent) before that iteration's solve, as
                          the paper's multi-corrector does */
-  int pdl;            /* 1 (default): the product kernels are launched with programmatic stream
-                         serialization: a product's CTAs start while the previous kernel drains,
-                         prefetch their own rows of the stored matrix into L2 and wait
-                         (griddepcontrol.wait) before reading any vector; 0: ordinary launches.
-                         Results are the same either way (measured: FP64 step 1084 -> 1069 ms,
-                         mixed 626 -> 615 ms on the 616k-node tube).
+  int pdl;            /* 1 (default): products of small and of large grids are launched with
+                         programmatic stream serialization: a product's CTAs start while the
+                         previous kernel drains, read their first rows of the stored matrix and
+                         wait (griddepcontrol.wait) before reading any vector; grids between half
+                         a CTA and eight CTAs per SM are slower that way and are launched plainly;
+                         0: ordinary launches.  Results are the same either way (measured: 1 % of
+                         an FP64 step on the 616k-node tube).
                          Like spmv_group and l2_prefetch it is process-wide: the last scr_create sets it */
   int tangent_resetup;/* how scr_assemble_tangent (and the Newton corrector) set the solve up on the
                          new tangent: 1 (default) scr_update_values (the aggregates, truncation

@@ -1245,47 +1245,53 @@ void to_dense(const DBsr<double>& A, double* dense, cudaStream_t s) {
 // exchanges the rows in its columns, scales row k and subtracts; column k
 // turns into the inverse's column.  The columns come out in the order of the
 // row exchanges and are put back at the end.
-// One CTA on [M | I] was bound by the FP64 pipe of one SM: 2 n^2 multiply-adds
-// per step at 2 a clock.  16 SMs on n^2 take (192 rows) 2.5 ms -> see
-// dense_inverse.
-__device__ __forceinline__ void invert_publish(const double* a, int k, int n, double* f, double* recip, int* piv,
-                                               int* singular, double* rv, int* ri) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  double best = -1.0;
-  int bi = k;
-  for (int r = k + tid; r < n; r += nt) {
-    const double v = fabs(a[r]);
-    if (v > best) {
-      best = v;
-      bi = r;
-    }
-  }
+// One CTA on [M | I] was bound by the FP64 pipe of one SM, 2 n^2 multiply-adds
+// per step at 2 a clock: the inverses of the small tube (192, 38 and 14 rows)
+// took 2.5 ms on average, with 16 SMs on n^2 and FP64 comparisons 0.73 ms.
+// The comparisons run on integers (non-negative doubles order like their bit
+// patterns): FP64 compares would queue on the FP64 pipe behind the updates.
+__device__ __forceinline__ long long pivot_key(double v) {  // -1: not a number
+  const long long b = __double_as_longlong(v) & 0x7fffffffffffffffLL;
+  return b > 0x7ff0000000000000LL ? -1 : b;
+}
+__device__ __forceinline__ void pivot_reduce(long long& best, int& bi) {
   for (int o = 16; o > 0; o >>= 1) {
-    const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+    const long long ov = __shfl_xor_sync(0xffffffffu, best, o);
     const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
     if (ov > best || (ov == best && oi < bi)) {
       best = ov;
       bi = oi;
     }
   }
+}
+__device__ __forceinline__ void invert_publish(const double* a, int k, int n, double* f, double* recip, int* piv,
+                                               int* singular, long long* rv, int* ri) {
+  const int tid = threadIdx.x, nt = blockDim.x, nw = nt >> 5;
+  long long best = -1;
+  int bi = n;
+  for (int r = k + tid; r < n; r += nt) {
+    const long long v = pivot_key(a[r]);
+    if (v > best) {
+      best = v;
+      bi = r;
+    }
+  }
+  pivot_reduce(best, bi);
   if ((tid & 31) == 0) {
     rv[tid >> 5] = best;
     ri[tid >> 5] = bi;
   }
   __syncthreads();
-  best = -1.0;
-  int p = k;
-  for (int w = 0; w < nt / 32; ++w)
-    if (rv[w] > best || (rv[w] == best && ri[w] < p)) {
-      best = rv[w];
-      p = ri[w];
-    }
+  best = (tid & 31) < nw ? rv[tid & 31] : -1;
+  bi = (tid & 31) < nw ? ri[tid & 31] : n;
+  pivot_reduce(best, bi);
+  const int p = best >= 0 ? bi : k;
   for (int r = tid; r < n; r += nt) f[r] = a[r == k ? p : r == p ? k : r];
   if (tid == 0) {
     const double d = a[p];
     *recip = d != 0.0 ? 1.0 / d : 0.0;
     *piv = p;
-    if (!(best > 0.0)) *singular = 1;
+    if (best <= 0) *singular = 1;
   }
 }
 
@@ -1299,10 +1305,10 @@ __global__ void __launch_bounds__(512) k_invert(double* M, double* Inv, int n, i
   double* recip = scratch + 2 * n;   // their pivots' reciprocals
   int* piv = reinterpret_cast<int*>(scratch + 2 * n + 2);
   double* f = sm;                    // the published column of this step
-  double* rv = sm + n;               // pivot search
+  long long* rv = reinterpret_cast<long long*>(sm + n);  // pivot search
   int* ri = reinterpret_cast<int*>(rv + nw);
   int* pos = ri + nw + (nw & 1);     // column order at the end (n)
-  double* cols = rv + nw + (nw + 1) / 2 + (n + 1) / 2;
+  double* cols = sm + n + nw + (nw + 1) / 2 + (n + 1) / 2;
   const int ncol = q < n ? (n - q + nc - 1) / nc : 0;
   auto column = [&](int lc) { return SM ? cols + (long long)lc * n : M + (long long)(q + lc * nc) * n; };
   if (SM) {
@@ -1328,7 +1334,8 @@ __global__ void __launch_bounds__(512) k_invert(double* M, double* Inv, int n, i
       __syncwarp();
       for (int r = lane; r < n; r += 32) {
         const double v = r == p ? ak : a[r], g = f[r];
-        a[r] = r == k ? t : g != 0.0 ? v - g * t : v;
+        const bool some = (__double_as_longlong(g) & 0x7fffffffffffffffLL) != 0;
+        a[r] = r == k ? t : some ? v - g * t : v;
       }
     }
     __syncthreads();
@@ -1357,9 +1364,8 @@ __global__ void __launch_bounds__(512) k_invert(double* M, double* Inv, int n, i
   }
 }
 
-// 16 CTAs of 512 threads (8 where the device places no cluster of 16).
-// Measured (us): see profiles of the set-up; shared memory holds the columns
-// up to about 560 rows, beyond that they stay in L2.
+// 16 CTAs of 512 threads (8 where the device places no cluster of 16); shared
+// memory holds the columns up to about 600 rows, beyond that they stay in L2.
 void dense_inverse(double* M, double* inv, int n, int* singular, cudaStream_t s) {
   if (n == 0) return;
   constexpr int kThreads = 512, kWarps = kThreads / 32;

@@ -1,5 +1,6 @@
-// Vector kernels of the Krylov solvers: deterministic two-stage reductions
-// (fixed grid, per-block partial sums reduced in a fixed order), the two
+// Vector kernels of the Krylov solvers: deterministic reductions (a grid fixed
+// by the length, per-CTA partial sums added in CTA order by the CTA that ends
+// last), the two
 // classical Gram-Schmidt passes of FGMRES/GMRES fused with their dot
 // products, Givens rotations of the Hessenberg least-squares problem on the
 // device, and the CG recurrences.

@@ -830,8 +830,8 @@ struct Hierarchy {
 // ------------------------------------------------------------ device loops
 // A GMRES solve can be recorded into a CUDA graph with its control flow on
 // the device (option graph_krylov): a WHILE node over the restart cycles
-// holds a WHILE node over the Arnoldi steps (copy of v_j, preconditioner,
-// operator, the Gram-Schmidt passes, the Givens update, v_{j+1}), then the
+// holds a WHILE node over the Arnoldi steps (preconditioner, operator, the
+// Gram-Schmidt passes with the Givens update, v_{j+1}), then the
 // solution update and an IF node with the restart.  One-thread kernels set
 // each node's condition from the residual estimate on the device, with the
 // same tests, in the same order, as the host-driven loop (Gmres::solve), so
