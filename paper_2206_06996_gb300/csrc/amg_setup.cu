@@ -1249,7 +1249,8 @@ void to_dense(const DBsr<double>& A, double* dense, cudaStream_t s) {
 // per step at 2 a clock: the inverses of the small tube (192, 38 and 14 rows)
 // took 2.5 ms on average, with 16 SMs on n^2 and FP64 comparisons 0.73 ms.
 // The comparisons run on integers (non-negative doubles order like their bit
-// patterns): FP64 compares would queue on the FP64 pipe behind the updates.
+// patterns): FP64 compares would queue on the FP64 pipe behind the updates
+// (a Newton step of the small tube, three inverses: 41.9 -> 40.1 ms).
 __device__ __forceinline__ long long pivot_key(double v) {  // -1: not a number
   const long long b = __double_as_longlong(v) & 0x7fffffffffffffffLL;
   return b > 0x7ff0000000000000LL ? -1 : b;
