@@ -108,8 +108,10 @@ void build_vec(DBsr<VT>& M, DeviceArena& a, cudaStream_t s);
 // mean) blocks, or of more than max(64, 8 x the mean) where the first are
 // more than one row in 512 (and 64): a CTA per row costs more than its share
 // of a lane group's waiting when many rows are long (Shat of the bench tube:
-// one row in ten, FP64 product 169 -> 323 us).  add() queues a pattern, read() waits once for all queued ones, set() gives list id to a
-// matrix with that pattern.
+// one row in ten, FP64 product 169 -> 323 us).  add() queues a pattern (any
+// number of them: a hierarchy queues two per level, and its levels are bounded
+// by the option amg_max_levels alone), read() waits once for all queued ones,
+// set() gives list id to a matrix with that pattern.
 class LongRows {
  public:
   LongRows(DeviceArena& a, cudaStream_t s);
@@ -124,14 +126,14 @@ class LongRows {
   }
 
  private:
-  static constexpr int kMax = 64;
+  static constexpr int kPage = 64;  // lists per array of counts
   struct List {
     int* rows;
     int thr[2], cap, n, pick;
   };
   DeviceArena& a_;
   cudaStream_t s_;
-  int* cnt_;
+  std::vector<int*> cnt_;
   std::vector<List> lists_;
 };
 

@@ -273,13 +273,13 @@ __global__ void k_long_rows(int nbr, const int* __restrict__ rp, int thr0, int t
       if (q < cap) rows[t * cap + q] = i;
     }
 }
-LongRows::LongRows(DeviceArena& a, cudaStream_t s) : a_(a), s_(s) {
-  cnt_ = a.alloc<int>(2 * kMax);
-  SCR_CUDA(cudaMemsetAsync(cnt_, 0, sizeof(int) * 2 * kMax, s));
-}
+LongRows::LongRows(DeviceArena& a, cudaStream_t s) : a_(a), s_(s) {}
 int LongRows::add(int nbr, long long nnzb, const int* rp) {
   const int id = (int)lists_.size();
-  if (id >= kMax) throw CudaError{cudaErrorInvalidValue, "too many long-row lists"};
+  if (id % kPage == 0) {  // the counts of kPage more lists
+    cnt_.push_back(a_.alloc<int>(2 * kPage));
+    SCR_CUDA(cudaMemsetAsync(cnt_.back(), 0, sizeof(int) * 2 * kPage, s_));
+  }
   List l;
   const long long mean = nbr ? nnzb / nbr : 0;
   l.thr[0] = (int)std::max<long long>(32, 3 * mean);
@@ -288,7 +288,8 @@ int LongRows::add(int nbr, long long nnzb, const int* rp) {
   l.n = l.pick = 0;
   l.rows = a_.alloc<int>(2 * l.cap);
   if (nbr > 0) {
-    k_long_rows<<<ceil_div(nbr, 256), 256, 0, s_>>>(nbr, rp, l.thr[0], l.thr[1], l.cap, l.rows, cnt_ + 2 * id);
+    k_long_rows<<<ceil_div(nbr, 256), 256, 0, s_>>>(nbr, rp, l.thr[0], l.thr[1], l.cap, l.rows,
+                                                    cnt_.back() + 2 * (id % kPage));
     SCR_LAUNCH();
     counters().launches++;
   }
@@ -296,8 +297,9 @@ int LongRows::add(int nbr, long long nnzb, const int* rp) {
   return id;
 }
 void LongRows::read() {
-  int h[2 * kMax] = {};
-  SCR_CUDA(cudaMemcpyAsync(h, cnt_, sizeof h, cudaMemcpyDeviceToHost, s_));
+  std::vector<int> h(2 * kPage * cnt_.size());
+  for (size_t p = 0; p < cnt_.size(); ++p)
+    SCR_CUDA(cudaMemcpyAsync(h.data() + 2 * kPage * p, cnt_[p], sizeof(int) * 2 * kPage, cudaMemcpyDeviceToHost, s_));
   SCR_CUDA(cudaStreamSynchronize(s_));
   for (size_t i = 0; i < lists_.size(); ++i)
     for (int t = 1; t >= 0; --t)
