@@ -189,7 +189,7 @@ struct Hierarchy {
   bool use_graph = false, graph_failed = false;
   GraphExecPtr gexec;
   void *gin = nullptr, *gout = nullptr;
-  size_t gsize = 0;  // element size the graph was captured for
+  size_t gsize = 0;  // element size of gin, gout and the graph
   long long glaunches = 0, gbytes = 0;
 
   int n_levels() const { return (int)lv.size(); }
@@ -397,10 +397,8 @@ struct Hierarchy {
   // the sparse products' patterns are those of the build (a numeric
   // re-set-up); the V-cycle graph is recorded again at its next use.
   void refresh(const DBsr<double>& A0, const scr_opts& o, cudaStream_t s, const DBsr<float>* A0f = nullptr) {
-    gexec.reset();
+    gexec.reset();  // its vectors gin and gout stay: sizes and precision are the build's
     graph_failed = false;
-    gin = gout = nullptr;
-    gsize = 0;
     const int nl = n_levels();
     if (nl == 0) return;
     settle(false);
@@ -741,8 +739,15 @@ struct Hierarchy {
   template <typename T>
   void capture(cudaStream_t s) {
     const long long n = lv[0].n * nrhs;
-    T* in = arena->alloc<T>(n + 1);
-    T* out = arena->alloc<T>(n + 1);
+    // the arena is given back by the next build only, and every numeric
+    // re-set-up records the graph again: the vectors are allocated once
+    if (!gin || gsize != sizeof(T)) {
+      gin = arena->alloc<T>(n + 1);
+      gout = arena->alloc<T>(n + 1);
+      gsize = sizeof(T);
+    }
+    T* in = input<T>();
+    T* out = output<T>();
     fill<T>(in, (T)0, n, s);
     // an eager V-cycle first: kernels configured on first use are set up
     // outside the capture
@@ -778,9 +783,6 @@ struct Hierarchy {
       return;
     }
     gexec.reset(ex);
-    gin = in;
-    gout = out;
-    gsize = sizeof(T);
   }
 
   // true when V-cycles are replayed from the recorded graph (recorded here at
