@@ -1369,14 +1369,16 @@ __global__ void __launch_bounds__(512) k_invert(double* M, double* Inv, int n, i
 // memory holds the columns up to about 600 rows, beyond that they stay in L2.
 void dense_inverse(double* M, double* inv, int n, int* singular, cudaStream_t s) {
   if (n == 0) return;
-  constexpr int kThreads = 512, kWarps = kThreads / 32;
+  constexpr int kThreads = 512, kWarps = kThreads / 32, kShared = 200 * 1024;
   const size_t head = sizeof(double) * (n + kWarps + (kWarps + 1) / 2 + (n + 1) / 2 + 2);
   for (int nc : {16, 8}) {
     const size_t cols = sizeof(double) * ((n + nc - 1) / nc) * (size_t)n;
-    const bool fits = head + cols <= 200 * 1024;
+    const bool fits = head + cols <= (size_t)kShared;
     const size_t bytes = fits ? head + cols : head;
     auto* kern = fits ? k_invert<true> : k_invert<false>;
-    SCR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    // the limit is the kernel's, in every thread: always the largest, or a
+    // smaller inverse in another thread would refuse this launch
+    SCR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kShared));
     if (nc > 8) SCR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nc);

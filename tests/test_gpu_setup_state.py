@@ -1,10 +1,12 @@
 """What set-ups leave behind and share: lists of long rows for any number of
-levels, device memory over numeric re-set-ups."""
+levels, device memory over numeric re-set-ups, set-ups of several threads."""
 import ctypes as C
 import os
 import shutil
 import subprocess
+import threading
 
+import numpy as np
 import pytest
 
 import fsi_inputs as F
@@ -64,3 +66,42 @@ def test_numeric_resetups_keep_the_device_memory(precision, loops):
             torch.cuda.synchronize()
             used.append(_pool_bytes())
     assert used[0] > 0 and used[1:] == used[:1] * 4
+
+
+def _dense(n, seed):
+    """A full matrix of n rows with a dominant diagonal, as 1x1 blocks."""
+    a = np.random.default_rng(seed).uniform(-1.0, 1.0, (n, n)) + 2.0 * n * np.eye(n)
+    return a, F.BSR(1, 1, n, n, np.arange(n + 1, dtype=np.int32) * n, np.tile(np.arange(n, dtype=np.int32), n),
+                    a.reshape(-1))
+
+
+def test_inverses_of_two_sizes_in_several_threads():
+    """Coarsest levels of 20 rows in six threads beside one of 560 rows,
+    inverted at once: the launch limits of one do not reach into another's (an
+    explicit inverse's residual is at most 8 n eps cond(A); cond < 4 here)."""
+    errors, done = [], threading.Event()
+
+    def work(n, times):
+        try:
+            a, L = _dense(n, n)
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream), pkg.BlockSolver(amg_max_levels=1, autotune=0) as sol:
+                b = torch.ones(3 * n, dtype=torch.float64, device="cuda")
+                for k in range(times):
+                    sol.mesh_setup(L)
+                    if n < 100 and done.is_set():
+                        break
+                x = sol.amg_apply(pkg.SCR_HIER_MESH, b).cpu().numpy().reshape(n, 3)
+            assert np.abs(a @ x - 1.0).max() <= 32 * n * np.finfo(float).eps * n
+        except Exception as e:  # noqa: BLE001 - reported below
+            errors.append(f"{n} rows: {e}")
+
+    small = [threading.Thread(target=work, args=(20, 20000)) for _ in range(6)]
+    large = threading.Thread(target=work, args=(560, 300))
+    for t in small + [large]:
+        t.start()
+    large.join()
+    done.set()
+    for t in small:
+        t.join()
+    assert not errors, errors
