@@ -175,6 +175,9 @@ void power_start_unit(double* v, long long n, const Reducer& red, double* nrm, c
 // the power iteration); the vector is normalised every fifth step, which
 // bounds its growth at lambda^5, and before the last step, whose norm is the
 // estimate.  Normalising every step cost six launches a step instead of one.
+// The squared norm then overflows from lambda of about 1e30 (a diagonal that
+// is almost zero beside its row): such an operator is iterated once more with
+// a normalisation per step, which bears lambda of 1e150.
 double power_lambda(const DBsr<double>& A, const double* dinv, int iters, cudaStream_t s) {
   const long long n = (long long)A.nbr * A.br;
   if (n == 0) return 0.0;
@@ -185,26 +188,29 @@ double power_lambda(const DBsr<double>& A, const double* dinv, int iters, cudaSt
   double* zero = tmp.alloc<double>(n);
   double* nrm = tmp.alloc<double>(2);
   fill<double>(zero, 0.0, n, s);
-  power_start_unit(v, n, red, nrm, s);
   EpiArgs e;
   e.kind = Epi::ScaledSub;
   e.z = zero;
   e.dinv = dinv;
-  for (int it = 0; it < iters; ++it) {
-    spmv<double, double>(A, v, w, 1, e, s);
-    std::swap(v, w);
-    if (it + 1 < iters && (it % 5 == 4 || it + 2 == iters)) {
-      norm2<double>(v, n, nrm, red, s);
-      k_rsqrt_scalar<<<1, 1, 0, s>>>(nrm, nrm + 1);
-      SCR_LAUNCH();
-      counters().launches++;
-      scale_by<double>(v, nrm + 1, v, n, s);
-    }
-  }
-  norm2<double>(v, n, nrm, red, s);
   double h = 0.0;
-  SCR_CUDA(cudaMemcpyAsync(&h, nrm, sizeof(double), cudaMemcpyDeviceToHost, s));
-  SCR_CUDA(cudaStreamSynchronize(s));
+  for (int every : {5, 1}) {
+    power_start_unit(v, n, red, nrm, s);
+    for (int it = 0; it < iters; ++it) {
+      spmv<double, double>(A, v, w, 1, e, s);
+      std::swap(v, w);
+      if (it + 1 < iters && (it % every == every - 1 || it + 2 == iters)) {
+        norm2<double>(v, n, nrm, red, s);
+        k_rsqrt_scalar<<<1, 1, 0, s>>>(nrm, nrm + 1);
+        SCR_LAUNCH();
+        counters().launches++;
+        scale_by<double>(v, nrm + 1, v, n, s);
+      }
+    }
+    norm2<double>(v, n, nrm, red, s);
+    SCR_CUDA(cudaMemcpyAsync(&h, nrm, sizeof(double), cudaMemcpyDeviceToHost, s));
+    SCR_CUDA(cudaStreamSynchronize(s));
+    if (h > 0.0 && std::isfinite(h)) break;
+  }
   return 1.1 * std::sqrt(h);
 }
 

@@ -1,5 +1,6 @@
 """What set-ups leave behind and share: lists of long rows for any number of
-levels, device memory over numeric re-set-ups, set-ups of several threads."""
+levels, device memory over numeric re-set-ups, set-ups of several threads; and set-ups
+of operators far from the usual scales."""
 import ctypes as C
 import os
 import shutil
@@ -10,6 +11,8 @@ import numpy as np
 import pytest
 
 import fsi_inputs as F
+from oracle import amg
+from oracle.sparse import to_csr
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -105,3 +108,26 @@ def test_inverses_of_two_sizes_in_several_threads():
     for t in small:
         t.join()
     assert not errors, errors
+
+
+@pytest.mark.parametrize("share", [1.0, 0.1])
+def test_vcycle_with_a_diagonal_next_to_zero_matches_oracle(share):
+    """Rows whose diagonal is 1e-36 of the others' entries give D^{-1} A an
+    eigenvalue of 1e36: its power iteration, the Chebyshev guard and the V-cycle
+    stay finite and equal the oracle's on the exported hierarchy (its V-cycle
+    moves by 2e-16 when its matrices do, so FP64 sums in another order stay
+    below 1e-10)."""
+    L = F.tube_system("tube_small").L
+    rows = np.repeat(np.arange(L.nb_rows), np.diff(L.row_ptr))
+    small = np.random.default_rng(1).random(L.nb_rows) < share
+    L.val[(L.col == rows) & small[rows]] *= 1e-36
+    with pkg.BlockSolver() as sol:
+        sol.mesh_setup(L)
+        nl = sol.amg_levels(pkg.SCR_HIER_MESH)
+        As = [to_csr(sol.export(pkg.SCR_HIER_MESH, l, pkg.SCR_EXPORT_OPERATOR)) for l in range(nl)]
+        Ps = [to_csr(sol.export(pkg.SCR_HIER_MESH, l, pkg.SCR_EXPORT_PROLONGATOR)) for l in range(nl - 1)]
+        b = np.random.default_rng(3).standard_normal(3 * L.nb_rows)
+        x = sol.amg_apply(pkg.SCR_HIER_MESH, torch.as_tensor(b, device="cuda")).cpu().numpy().reshape(-1, 3)
+    assert nl > 1
+    ref = amg.vcycle(amg.hierarchy_from_matrices(As, Ps, 1, 1, 1, "cheb", 3), b.reshape(-1, 3))
+    assert np.all(np.isfinite(x)) and np.linalg.norm(x - ref) <= 1e-10 * np.linalg.norm(ref)
