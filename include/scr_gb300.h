@@ -114,7 +114,7 @@ typedef struct {
   int sell;           /* 0: slab products; W > 0: products with A, Shat and L use a sliced block-ELL
                          copy with rows sorted by length inside windows of W block rows
                          (W a multiple of 32, at most 1024); default 0 */
-  int vec;            /* 1 (default): A and Shat (and their FP32 copies) also keep a padded copy in
+  int vec;            /* 1 (default): A and Shat (in mixed precision their FP32 copies) also keep a padded copy in
                          which every block row's column indices and scalar rows start on 16-byte
                          boundaries (zero padding), and the autotuner also times the kernels that
                          read it with 16-byte vector loads; 0: slab products only */

@@ -137,6 +137,13 @@ class LongRows {
   std::vector<List> lists_;
 };
 
+// M for the products of the smoother's set-up (power iteration, Chebyshev
+// guard), one right-hand side: with a kernel that its sizes choose, not the
+// timed one.  The timed choice differs between processes, and with it the
+// order of the sums: lambda moved by an ulp, and a guard value next to its
+// limit could change a level's smoother.
+DBsr<double> setup_product(const DBsr<double>& M);
+
 // forced kernel code for every product (0: per-matrix choice)
 void set_forced_group(int code);
 int forced_group();

@@ -280,7 +280,7 @@ struct Hierarchy {
       break;
     }
     // long rows of the levels' operators and restrictions (before the smoother
-    // data, whose products a numeric re-set-up runs in the same way)
+    // data, whose products use them, as a numeric re-set-up's do)
     {
       LongRows lr(ar, s);
       std::vector<int> ia(lv.size(), -1), ir(lv.size(), -1);
@@ -294,7 +294,7 @@ struct Hierarchy {
         lr.set(ir[l], lv[l].R);
       }
     }
-    // product kernels of the FP64 levels, before the smoother data (as above)
+    // product kernels of the FP64 levels' V-cycles
     if (o.autotune && !f32)
       for (size_t l = 0; l + 1 < lv.size(); ++l) {
         Level& L = lv[l];
@@ -331,8 +331,9 @@ struct Hierarchy {
       if (smoother == SCR_SMOOTH_CHEB && l + 1 < lv.size()) {
         L.dd = ar.alloc<double>(L.n + 1);
         inv_diag(L.A, L.dd, s);
-        L.lam = power_lambda(L.A, L.dd, 20, s);
-        L.cheb_off = cheb_guard_growth(L, s) > kChebGuardGrowth;
+        const DBsr<double> Ms = setup_product(L.A);
+        L.lam = power_lambda(Ms, L.dd, 20, s);
+        L.cheb_off = cheb_guard_growth(Ms, L, s) > kChebGuardGrowth;
         if (o.verbose && L.cheb_off)
           fprintf(stderr, "[amg bs=%d] level %zu: Chebyshev guard -> l1-Jacobi\n", bs, l);
         if (f32) {
@@ -448,8 +449,9 @@ struct Hierarchy {
       Level& L = lv[l];
       if (smoother == SCR_SMOOTH_CHEB && l + 1 < nl) {
         inv_diag(L.A, L.dd, s);
-        L.lam = power_lambda(L.A, L.dd, 20, s);
-        L.cheb_off = cheb_guard_growth(L, s) > kChebGuardGrowth;
+        const DBsr<double> Ms = setup_product(L.A);
+        L.lam = power_lambda(Ms, L.dd, 20, s);
+        L.cheb_off = cheb_guard_growth(Ms, L, s) > kChebGuardGrowth;
         if (f32) cast_d2f(L.dd, L.ddf, L.n, s);
       }
       if (f32) {
@@ -511,7 +513,7 @@ struct Hierarchy {
   // eigenvalues of D^{-1}A off [lam/30, lam], where the polynomial amplifies.
   static constexpr int kChebGuardSweeps = 5;
   static constexpr double kChebGuardGrowth = 10.0;
-  double cheb_guard_growth(Level& L, cudaStream_t s) {
+  double cheb_guard_growth(const DBsr<double>& A, const Level& L, cudaStream_t s) {
     const long long n = L.n;
     DeviceArena tmp(s);
     Reducer red = make_reducer(tmp);
@@ -536,7 +538,7 @@ struct Hierarchy {
       f.dinv = L.dd;
       f.r = r;
       f.dout = d0;
-      spmv<double, double>(L.A, e, out, 1, f, s);
+      spmv<double, double>(A, e, out, 1, f, s);
       double *a = d0, *b = d1;
       EpiArgs g;
       g.kind = Epi::ChebStep;
@@ -547,7 +549,7 @@ struct Hierarchy {
         g.beta = ab.second;
         g.dout = b;
         g.xsol = out;
-        spmv<double, double>(L.A, a, b, 1, g, s);
+        spmv<double, double>(A, a, b, 1, g, s);
         std::swap(a, b);
       }
       std::swap(e, out);
@@ -1977,7 +1979,7 @@ int scr_setup(scr_handle h, const scr_bsr* A, const scr_bsr* B, const scr_bsr* C
       build_sell<double>(h->Shat, h->Shat_sell, a, s, h->o.sell);
       h->Shat.sell = &h->Shat_sell;
     }
-    if (h->o.vec) {
+    if (h->o.vec && !f32) {  // in mixed precision the solve reads the FP32 copies'
       build_vec<double>(h->A, a, s);
       build_vec<double>(h->Shat, a, s);
     }
@@ -1989,9 +1991,10 @@ int scr_setup(scr_handle h, const scr_bsr* A, const scr_bsr* B, const scr_bsr* C
     lr.set(lS, h->Shat);
     lr.set(lB, h->B);
     lr.set(lC, h->C);
-    tune_product<double>(h->A, h->k, h->o, a, s);
-    tune_product<double>(h->Shat, h->k, h->o, a, s);
-    if (f32) {
+    if (!f32) {
+      tune_product<double>(h->A, h->k, h->o, a, s);
+      tune_product<double>(h->Shat, h->k, h->o, a, s);
+    } else {
       h->Af = float_copy(h->A, a, s);
       if (h->o.vec) build_vec<float>(h->Af, a, s);
       h->Bf = float_copy(h->B, a, s);

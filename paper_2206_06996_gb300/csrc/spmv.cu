@@ -560,6 +560,28 @@ void tune_load(const char* path) {
   for (const auto& kv : got) tune_cache()[kv.first] = kv.second;
 }
 
+// The rule by row length (pick_group) with wider groups where they were
+// faster, so that the products stay within a few per cent of the best timed
+// ones (us per Chebyshev step; pick_group's own choice in brackets): 3x3, 15
+// blocks a row, 616k rows: 401 181 (211), 95k rows 34.9 (39.5), at 47k rows 27.2
+// (26.3), 5.9k rows: 104 8.3 (10.0), at 10.8k rows 10.8 (10.8); 1x1, 80 entries a
+// row, 655k rows: 104 164 (220), 60k rows of 49: 16.9 (20.6), 6.9k rows of 70: 108
+// 8.7 (11.2); 1x1, 22 entries, 69k rows: 102 21.4 (26.8).
+DBsr<double> setup_product(const DBsr<double>& M) {
+  DBsr<double> S = M;
+  S.g = 0;
+  if (M.nbr == 0) return S;
+  int G = pick_group(S);
+  const double per_row = (double)M.nnzb * M.bc / M.nbr;
+  if (M.br == 3 && M.bc == 3) {
+    if (M.nbr < 8192 && per_row >= 24) G = std::max(G, 4);
+  } else if (per_row >= 16) {
+    G = std::max(G, per_row < 32 ? 2 : per_row >= 64 && M.nbr < 8192 ? 8 : 4);
+  }
+  S.g = M.br == 3 && M.bc == 3 && M.nbr >= 65536 ? 401 : 100 + G;
+  return S;
+}
+
 template int autotune_spmv<double>(DBsr<double>&, int, cudaStream_t);
 template int autotune_spmv<float>(DBsr<float>&, int, cudaStream_t);
 

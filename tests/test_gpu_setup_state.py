@@ -1,6 +1,6 @@
 """What set-ups leave behind and share: lists of long rows for any number of
-levels, device memory over numeric re-set-ups, set-ups of several threads; and set-ups
-of operators far from the usual scales."""
+levels, device memory over numeric re-set-ups, set-ups of several threads, set-ups with
+other timed kernels; and set-ups of operators far from the usual scales."""
 import ctypes as C
 import os
 import shutil
@@ -131,3 +131,43 @@ def test_vcycle_with_a_diagonal_next_to_zero_matches_oracle(share):
     assert nl > 1
     ref = amg.vcycle(amg.hierarchy_from_matrices(As, Ps, 1, 1, 1, "cheb", 3), b.reshape(-1, 3))
     assert np.all(np.isfinite(x)) and np.linalg.norm(x - ref) <= 1e-10 * np.linalg.norm(ref)
+
+
+def test_smoother_data_do_not_depend_on_the_timed_kernels(tmp_path):
+    """Set-ups (and numeric re-set-ups) with two files of product kernels hold
+    the same smoother data: V-cycles of all hierarchies, run with one forced
+    kernel, are bit-identical."""
+    s = F.tube_system("tube_small")
+    with pkg.BlockSolver() as sol:  # every pattern is in the table
+        sol.setup(s.A, s.B, s.C, s.D)
+        sol.mesh_setup(s.L)
+    pkg.tune_save(str(tmp_path / "timed.txt"))
+    lines = (tmp_path / "timed.txt").read_text().splitlines()
+    for name, codes in (("one", ("101", "101")), ("two", ("402", "104"))):
+        rows = [l.split() for l in lines if not l.startswith("#")]
+        text = "".join(" ".join(r[:7] + [codes[0] if r[3] == "3" else codes[1]]) + "\n" for r in rows)
+        (tmp_path / name).write_text(text)
+    rng = np.random.default_rng(2)
+    b = {w: torch.as_tensor(rng.standard_normal(n), device="cuda")
+         for w, n in ((pkg.SCR_HIER_A, 3 * s.n_v), (pkg.SCR_HIER_SHAT, s.n_p), (pkg.SCR_HIER_MESH, 3 * s.L.nb_rows))}
+    sols = []
+    try:
+        for name in ("one", "two"):
+            pkg.tune_load(str(tmp_path / name))
+            sols.append(pkg.BlockSolver().setup(s.A, s.B, s.C, s.D))
+            sols[-1].mesh_setup(s.L)
+        assert [x.stats()["kernel_A"] for x in sols] == [101, 402]
+        for again in range(2):
+            if again:
+                pkg.BlockSolver().close()  # no forced kernel
+                for x in sols:
+                    x.update_values(s.A, s.B, s.C, s.D)
+            pkg.BlockSolver(spmv_group=102).close()  # forces every product's kernel from here
+            for which, rhs in b.items():
+                one, two = (x.amg_apply(which, rhs).cpu().numpy() for x in sols)
+                np.testing.assert_array_equal(one, two)
+    finally:
+        pkg.tune_load(str(tmp_path / "timed.txt"))
+        pkg.BlockSolver().close()
+        for x in sols:
+            x.close()
