@@ -477,8 +477,8 @@ int scr_profile_end(scr_handle h, scr_kprof* out);
 
 /* The autotuner's kernel choices (scr_opts.autotune) live in a process-wide
    cache keyed by block shape, block rows and columns, stored blocks, value
-   precision (plus whether the matrix has the padded 16-byte copy of the
-   vec option) and right-hand sides.  scr_tune_save writes every cached
+   precision (BF16 copies apart; plus whether the matrix has the padded
+   16-byte copy of the vec option) and right-hand sides.  scr_tune_save writes every cached
    decision to a text file, one per line; scr_tune_load adds the decisions of
    such a file to the cache for the current device, so later set-ups of
    matrices with those keys skip the timing and use the stored kernels.  Use:

@@ -414,8 +414,10 @@ int autotune_spmv(DBsr<VT>& M, int nrhs, cudaStream_t s) {
   if (M.nbr == 0 || M.sell) return M.g;
   int dev = 0;
   cudaGetDevice(&dev);
-  // value bytes, plus 100 when M has the padded 16-byte copy (its candidates differ)
-  const TuneKey key{M.nnzb, M.nbr, M.nbc, M.br, M.bc, (int)sizeof(VT) + (M.vdesc ? 100 : 0), nrhs, dev};
+  // value bytes, plus 100 when M has the padded 16-byte copy (its candidates
+  // differ), plus 200 when its products read BF16 values (other kernels)
+  const TuneKey key{M.nnzb, M.nbr, M.nbc, M.br, M.bc, (int)sizeof(VT) + (M.vdesc ? 100 : 0) + (M.hval ? 200 : 0), nrhs,
+                    dev};
   {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     auto it = tune_cache().find(key);
@@ -516,7 +518,8 @@ int autotune_spmv(DBsr<VT>& M, int nrhs, cudaStream_t s) {
   return bestg;
 }
 // text form of the cache: "nnzb nbr nbc br bc value_bytes nrhs code" per line
-// (value_bytes + 100 for matrices with the padded 16-byte copy)
+// (value_bytes + 100 for matrices with the padded 16-byte copy, + 200 for
+// those whose products read BF16 values)
 static bool valid_code(int c) {
   return (c >= 1 && c <= 16) || (c >= 101 && c <= 116) || (c >= 301 && c <= 316) ||
          (c >= 401 && c <= 416);

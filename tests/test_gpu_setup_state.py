@@ -1,6 +1,7 @@
 """What set-ups leave behind and share: lists of long rows for any number of
 levels, device memory over numeric re-set-ups, set-ups of several threads, set-ups with
-other timed kernels; and set-ups of operators far from the usual scales."""
+other timed kernels, timed kernels of BF16 levels; and set-ups of operators far
+from the usual scales."""
 import ctypes as C
 import os
 import shutil
@@ -171,3 +172,18 @@ def test_smoother_data_do_not_depend_on_the_timed_kernels(tmp_path):
         pkg.BlockSolver().close()
         for x in sols:
             x.close()
+
+
+def test_levels_with_bf16_values_have_timed_kernels_of_their_own(tmp_path):
+    """Coarse levels of the same sizes with BF16 and with FP32 values run
+    different kernels: the table of timed choices holds an entry for each
+    (value bytes 4, and 204 with BF16 values)."""
+    s = F.tube_system("tube_small")
+    for bf16 in (1, 0):
+        with pkg.BlockSolver(precision=pkg.SCR_MIXED, amg_coarse_bf16=bf16) as sol:
+            sol.setup(s.A, s.B, s.C, s.D)
+            P1 = sol.export(pkg.SCR_HIER_A, 1, pkg.SCR_EXPORT_PROLONGATOR)
+    pkg.tune_save(str(tmp_path / "t.txt"))
+    rows = [l.split() for l in (tmp_path / "t.txt").read_text().splitlines() if not l.startswith("#")]
+    key = [str(v) for v in (len(P1.col), P1.nb_rows, P1.nb_cols, 3, 3)]
+    assert {r[5] for r in rows if r[:5] == key and r[6] == "1"} >= {"4", "204"}
