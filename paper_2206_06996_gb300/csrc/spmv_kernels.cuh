@@ -695,20 +695,11 @@ __global__ void __launch_bounds__(256) k_sell_spmv(DSell<VT> S, const XT* __rest
 // forced kernel code of every product (0: per matrix); defined in spmv.cu
 extern int g_l2_prefetch;
 
-// Grids of at most half a CTA per SM, or of at least eight per SM, are launched
-// early (pdl).  A chain of products of sizes between is slower that way: the
-// next kernel's waiting CTAs take slots, and the last CTAs of this one and the
-// first of the next fill the SMs unevenly.  Measured (us per product in a chain, plain / early): FP64, 2
-// lanes, 6000 rows 5.0 / 8.2, 50,000 rows 18.0 / 18.2; FP32, 4 lanes 2.8 / 4.3
-// and 9.9 / 9.8; FP32, 300 rows 2.4 / 2.3; at the bench tube's size early
-// launches take 1 % off an FP64 step.
-constexpr long long kEarlyMost = 76, kEarlyLeast = 8 * 152;
-
 // the product kernels' launch: the long rows' CTAs first, then those of args
 template <typename VT, typename... KArgs, typename... Args>
 inline void launch_rows(const DBsr<VT>& M, void (*kern)(KArgs...), long long ctas, cudaStream_t s, Args... args) {
   const long long grid = ctas + M.nlong;
-  launch_early(M.settled && (grid <= kEarlyMost || grid >= kEarlyLeast), kern, grid, 256, s, args..., M.lrow, M.nlong,
+  launch_early(M.settled && early_grid(grid, sm_count()), kern, grid, 256, s, args..., M.lrow, M.nlong,
                M.lthr);
 }
 
