@@ -43,13 +43,15 @@ def test_long_row_lists_of_more_patterns_than_a_page(tmp_path):
     assert r.returncode == 0 and r.stdout == "ok\n", r.stdout + r.stderr
 
 
-def _pool_bytes(attr=7):
+def _pool_bytes(attr=7, reset=False):
     """Bytes in use in the device's memory pool, which the library allocates
     from (attribute 7: current, 8: the highest since it was last reset)."""
     path = next(l.split()[-1] for l in open("/proc/self/maps") if "libcudart" in l)
     rt = C.CDLL(path)
     pool, v = C.c_void_p(), C.c_uint64()
     assert rt.cudaDeviceGetDefaultMemPool(C.byref(pool), torch.cuda.current_device()) == 0
+    if reset:
+        assert rt.cudaMemPoolSetAttribute(pool, attr, C.byref(v)) == 0
     assert rt.cudaMemPoolGetAttribute(pool, attr, C.byref(v)) == 0
     return v.value
 
@@ -187,3 +189,20 @@ def test_levels_with_bf16_values_have_timed_kernels_of_their_own(tmp_path):
     rows = [l.split() for l in (tmp_path / "t.txt").read_text().splitlines() if not l.startswith("#")]
     key = [str(v) for v in (len(P1.col), P1.nb_rows, P1.nb_cols, 3, 3)]
     assert {r[5] for r in rows if r[:5] == key and r[6] == "1"} >= {"4", "204"}
+
+
+def test_only_the_16_byte_kernels_build_a_padded_copy():
+    """A product with a forced kernel builds what that kernel reads: triples of
+    lanes (401) hold no more than the scalar-row kernel (101), the 16-byte
+    kernels (304) their padded copy beside it."""
+    A = pkg.DeviceBSR.from_host(F.tube_system("tube_small").A)
+    x = torch.ones(3 * A.nb_cols, dtype=torch.float64, device="cuda")
+    peak = {}
+    for code in (101, 401, 304):
+        with pkg.BlockSolver(spmv_group=code, autotune=0):
+            low = _pool_bytes(8, reset=True)
+            pkg.bsr_spmv(A, x)
+            peak[code] = _pool_bytes(8) - low
+    pkg.BlockSolver().close()  # no forced kernel from here
+    values = 8 * 9 * A.nnzb
+    assert values <= peak[101] < 1.5 * values and peak[401] == peak[101] and peak[304] > 2 * values
