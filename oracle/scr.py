@@ -27,7 +27,7 @@ infrastructure only; the CPU reference of the whole solver path).
 * Fixed-count A solves (options inner_vcycles, inter_vcycles): the paper's
   inner and intermediate solves are GMRES to a tolerance; with k > 0 they are
   k V-cycle-preconditioned Richardson steps instead, a fixed linear operator
-  (valid under the flexible outer FGMRES; the reading is stated in DESIGN).
+  (valid under the flexible outer FGMRES).
 """
 from __future__ import annotations
 

@@ -62,7 +62,7 @@ struct DBsr {
   // stay as they are until the next set-up: a product launched while its
   // predecessor drains may read them before it waits (pdl)
   bool settled = false;
-  // rows of more than lthr blocks (build_long_rows), which a product gives a
+  // rows of more than lthr blocks (LongRows), which a product gives a
   // CTA each
   const int* lrow = nullptr;
   int nlong = 0, lthr = 0x7fffffff;

@@ -7,10 +7,10 @@
 // itself, so a completed predecessor means that all earlier ones completed.
 // Launched without the attribute, both instructions return at once.
 //
-// The assembler and the compiler may move loads through the read-only path
-// (__ldg, const __restrict__ arguments) across the wait.  So a kernel reads
-// that way only what no kernel in flight may write (settled matrices), and
-// vectors with ordinary loads behind the wait.
+// Nothing orders loads through the read-only path (__ldg, const __restrict__
+// arguments) behind the wait.  As a precaution a kernel reads that way only
+// what no kernel in flight may write (settled matrices), and vectors with
+// ordinary loads behind the wait.
 #pragma once
 #include "common.cuh"
 

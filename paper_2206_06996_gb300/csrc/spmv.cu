@@ -1,13 +1,16 @@
 // Block-sparse matrix-vector products (slab layout), layout conversions and
 // the fused 2x2 block operator calA = [[A, B], [C, D]] of Sec. 5.2.1.
 //
-// Work decomposition: one group of G lanes per SCALAR row.  A scalar row of
-// a block row is contiguous in the slab layout (k*BC values), so the G lanes
-// stream it with one multiply-add per stored value and combine their partial
-// sums with log2(G) shuffles.  G is small (2-8): on GB300 the FP64 pipe
-// (about two FP64 FMAs per SM clock) is the binding resource of an FP64
-// SpMV, and a wider group would spend more FP64 adds on the cross-lane
-// reduction than on the product itself.
+// Work decomposition, general form: one group of G lanes per SCALAR row.  A
+// scalar row of a block row is contiguous in the slab layout (k*BC values), so
+// the G lanes stream it with one multiply-add per stored value and combine
+// their partial sums with log2(G) shuffles.  G is small (2-8): on GB300 the
+// FP64 pipe (about two FP64 FMAs per SM clock) is the binding resource of an
+// FP64 SpMV, and a wider group would spend more FP64 adds on the cross-lane
+// reduction than on the product itself.  Beside it, chosen by timing: triples
+// of lanes per block row of 3x3 blocks, lane groups per block row with 16-byte
+// loads on a padded copy (A and Shat); by rule: a CTA per long row, 16 bytes of
+// columns per lane for eight right-hand sides (spmm.cu).
 #include <cuda_bf16.h>
 
 #include <cstdarg>
@@ -476,7 +479,6 @@ int autotune_spmv(DBsr<VT>& M, int nrhs, cudaStream_t s) {
   }
   float best = 1e30f;
   int bestg = M.g;
-  const int saved = M.g;
   float times[16] = {};
   for (int q = 0; q < ncand; ++q) {
     const int code = cands[q];
@@ -496,7 +498,6 @@ int autotune_spmv(DBsr<VT>& M, int nrhs, cudaStream_t s) {
       bestg = code;
     }
   }
-  (void)saved;
   M.settled = was_settled;
   counters().launches += 6 * ncand;
   cudaEventDestroy(e0);

@@ -153,8 +153,9 @@ __device__ __forceinline__ void long_row_cta(int i, const int* __restrict__ rp, 
   }
 }
 
-// Rows of more than two rounds of their group are summed by the whole warp
-// (the block operator and Algorithm 2's last line, whose rows span matrices).
+// Rows of more than two rounds of their group (eight rounds of one-column
+// blocks), and of more than 32 blocks, are summed by the whole warp (the block
+// operator and Algorithm 2's last line, whose rows span matrices).
 template <int BC, int G, int U>
 constexpr int kLongRow = (BC == 3 ? 2 : 8) * G * U > 32 ? (BC == 3 ? 2 : 8) * G * U : 32;
 
@@ -530,8 +531,8 @@ struct Chunk33 {
 // chunks of V blocks in turn and accumulates all three scalar rows, so a
 // block's column index and its three source values are loaded once for its 9
 // multiply-adds.  The three row sums are combined over the G lanes and
-// written by lanes 0, 1, 2 (mod G).  Rows of more than two chunks per lane are
-// summed by the whole warp; loads before the wait as in k_spmv.
+// written by lanes 0, 1, 2 (mod G).  Rows of more than lthr blocks are the CTAs'
+// of long_row_cta; loads before the wait as in k_spmv.
 template <int G, typename VT, typename XT, Epi E>
 __global__ void __launch_bounds__(256, sizeof(VT) == 4 ? 4 : 3) k_spmv_vec33(int nbr, const int4* __restrict__ desc, const int* __restrict__ col,
                                                     const VT* __restrict__ val, const XT* x,
