@@ -108,10 +108,13 @@ def peaks():
 FP64_FMA_PER_SM_CLK = 2
 N_SM = 152
 # dram bytes / algorithmic bytes of the level-0 A products, from one ncu
-# capture each of the scalar-row kernel with the Chebyshev-step epilogue on
-# the 309k-node tube (2 lanes per scalar row; FP64 396.7 / 403.6 MB, FP32
-# 206.5 / 211.4 MB: see profiles/)
-TRAFFIC_RATIO = {"fp64": 396.7 / 403.6, "fp32": 206.5 / 211.4}
+# capture each with the Chebyshev-step epilogue on the 309k-node tube: the
+# scalar-row kernel with 2 lanes (codes 0 and 102; FP64 396.7 / 403.6 MB, FP32
+# 206.5 / 211.4 MB) and one triple of lanes per block row (code 401; 411.0 and
+# 206.7 MB): see profiles/
+TRAFFIC_RATIO = {"fp64": 396.7 / 403.6, "fp32": 206.5 / 211.4,
+                 "fp64 triples": 411.0 / 403.6, "fp32 triples": 206.7 / 211.4}
+CAPTURED_CODES = {0: "", 102: "", 401: " triples"}
 
 
 class ClockSampler:
@@ -247,11 +250,12 @@ def roofline(kprof: dict | None, fp64: bool, clocks: dict, ms_step: float, hbm: 
     if roof is None:
         roof = {"bound": "hbm", "achieved": achieved_gbs, "peak": hbm, "unit": "GB/s", "frac": achieved_gbs / hbm,
                 "peak_note": f"{peak_kind} HBM copy bandwidth (MEASURED_PEAKS.json hbm_gbs)"}
-    ratio = TRAFFIC_RATIO["fp64" if fp64 else "fp32"]
+    which = CAPTURED_CODES.get(kernel_code) if captured else None
+    ratio = None if which is None else TRAFFIC_RATIO[("fp64" if fp64 else "fp32") + which]
     roof.update({"kernel": kernel, "kernel_code": kernel_code, "launches_per_step": kprof["launches"],
                  "timed_launches": kprof["timed"], "bytes_per_launch": bytes_pl, "us_per_launch": per_launch_s * 1e6,
                  "share_of_step": kprof["ms"] / ms_step,
-                 "traffic": ratio * bytes_pl if (captured and ratio and kernel_code in (0, 102)) else None})
+                 "traffic": ratio * bytes_pl if ratio else None})
     if roof["traffic"] is not None:
         roof["traffic_note"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of the same kernel on a smaller tube, "
                                 "scaled to this launch by its algorithmic bytes")

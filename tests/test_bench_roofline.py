@@ -67,3 +67,12 @@ def test_traffic_ratios_are_the_captured_ones():
     # dram read + write over algorithmic bytes of the captured Chebyshev-step launches
     assert bench.TRAFFIC_RATIO["fp64"] == pytest.approx(396.7 / 403.6)
     assert bench.TRAFFIC_RATIO["fp32"] == pytest.approx(206.5 / 211.4)
+
+
+@pytest.mark.parametrize("fp64,dram,algorithmic", [(True, 411.0, 403.6), (False, 206.7, 211.4)])
+def test_traffic_of_the_triples_of_lanes_is_the_captured_one(fp64, dram, algorithmic):
+    kp = _kprof(181.0 if fp64 else 82.0, 782.86e6, 2.0 * 9 * BLOCKS)
+    r = bench.roofline(kp, fp64, CLOCKS, 850.0, HBM, "measured", "A", 401)
+    assert r["traffic"] == pytest.approx(dram / algorithmic * 782.86e6) and "smaller tube" in r["traffic_note"]
+    assert bench.roofline(kp, fp64, CLOCKS, 850.0, HBM, "measured", "A", 401, captured=False)["traffic"] is None
+    assert bench.roofline(kp, fp64, CLOCKS, 850.0, HBM, "measured", "A", 402)["traffic"] is None
